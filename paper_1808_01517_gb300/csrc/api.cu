@@ -280,6 +280,10 @@ static delimit_status check_device(int device) {
   cudaError_t e = cudaGetDevice(&cur);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
   if (cur != device) return fail(DELIMIT_ERR_INVALID_ARG, "handle was created on another device than the current one");
+  // binds the device's primary context to a thread that has made no CUDA call yet (autograd's
+  // backward thread, for instance): encoding a tensor map needs it
+  e = cudaSetDevice(cur);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
   return DELIMIT_OK;
 }
 
