@@ -117,6 +117,7 @@ struct delimit_lsc_geometry {
   LscDims dims_template;  // without channel counts
   FusedTables fused;      // B_s^T of the output basis for the LSC forward with SH2Signal fused
   BuildWTables bw;        // BF16 parts of M for the tensor-core operator build
+  ReduceDwTables rd;      // BF16 parts of M for the weight gradient's tensor-core reduction
 };
 
 static std::vector<double> transpose(const std::vector<double>& a, int rows, int cols) {
@@ -532,6 +533,13 @@ delimit_status delimit_lsc_geometry_create(const delimit_sh_basis* ob, int order
       delete g;
       return fail(DELIMIT_ERR_OOM, "operator-build tables: " + ferr);
     }
+    if (reduce_dw_tables_create(g->dims_template, g->d_M, g->rd, ferr) != cudaSuccess) {
+      build_w_tables_destroy(g->bw);
+      fused_tables_destroy(g->fused);
+      cudaFree(g->d_mem);
+      delete g;
+      return fail(DELIMIT_ERR_OOM, "weight-gradient reduction tables: " + ferr);
+    }
     g->on_device = true;
   }
   *out = g;
@@ -547,6 +555,7 @@ delimit_status delimit_lsc_geometry_destroy(delimit_lsc_geometry* g) {
     cudaFree(g->d_mem);
     fused_tables_destroy(g->fused);
     build_w_tables_destroy(g->bw);
+    reduce_dw_tables_destroy(g->rd);
     if (cur != g->device && cur >= 0) cudaSetDevice(cur);
   }
   delete g;
@@ -1028,8 +1037,13 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* s
       e = launch_wgrad_simt(a, d.s_out, per_out, maxN, p.splits, int(act_t), cs);
       if (e != cudaSuccess) return cuda_fail(e, "LSC weight-gradient launch");
     }
-    e = launch_reduce_dw(d, P, p_rs, p_cs, split_stride, p.splits, g->d_M, g->d_Mt, g->d_q, dw, db,
-                         reinterpret_cast<float*>(base + p.off_dwp), cs);
+    float* dwp = reinterpret_cast<float*>(base + p.off_dwp);
+    // BF16 activations: the reduction on the tensor cores (its error, that of an FP32 sum, is far
+    // below the voxel sums'); FP32 ones keep FP32 FMAs
+    if (act_t == DELIMIT_BF16 && tc && tc_reduce_dw_supported(g->rd))
+      e = tc_reduce_dw(d, g->rd, P, p_cs, split_stride, p.splits, g->d_q, dw, db, dwp, g->err_word, cs);
+    else
+      e = launch_reduce_dw(d, P, p_rs, p_cs, split_stride, p.splits, g->d_M, g->d_Mt, g->d_q, dw, db, dwp, cs);
     if (e != cudaSuccess) return cuda_fail(e, "dw/db reduction launch");
   }
   return DELIMIT_OK;

@@ -101,6 +101,22 @@ void build_w_tables_destroy(BuildWTables& t);
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t);
 cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, void* W, int* err, cudaStream_t st);
 
+// Parts of the collapse matrices for the weight gradient's reduction on the tensor cores: per
+// shell (or shell pair) and input coefficient b the three BF16 parts of M as operand images (ok
+// false: more than 64 kernel points or tables that do not fit; the CUDA-core reduction runs).
+struct ReduceDwTables {
+  void* d_img = nullptr;
+  int npg = 0;
+  bool ok = false;
+};
+cudaError_t reduce_dw_tables_create(const LscDims& dims_template, const float* d_M, ReduceDwTables& t,
+                                    std::string& err);
+void reduce_dw_tables_destroy(ReduceDwTables& t);
+bool tc_reduce_dw_supported(const ReduceDwTables& t);
+// dw and db as launch_reduce_dw from the transposed partials; scratch: reduce_dw_scratch_floats(d)
+cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float* P, int64_t ldpt, int64_t split_stride,
+                         int splits, const float* q, float* dw, float* db, float* scratch, int* err, cudaStream_t st);
+
 struct FusedTables {
   void* d_b2 = nullptr;
   int shells = 0, m[4] = {}, dir_off[4] = {};

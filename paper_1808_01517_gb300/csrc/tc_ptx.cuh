@@ -236,6 +236,49 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       : "memory");
 }
 
+// the same with A read from TMEM: 128 lanes (rows) x 8 columns of two BF16 K elements each
+// (the even one in the low half) per 16-deep MMA
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// 32 lanes x 8 consecutive 32-bit columns from registers; tmem_wait_st() before another thread
+// is told of them
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// (x, y) -> BF16 parts packed in pairs: x = x0 + x1 + x2 and y likewise, each part the
+// round-to-nearest BF16 of what the earlier ones leave (the differences are exact in FP32);
+// p[q] holds part q of x in its low and of y in its high half
+__device__ __forceinline__ void split3x2(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    p[q] = *reinterpret_cast<const uint32_t*>(&h);
+    if (q < 2) {
+      x -= __uint_as_float(p[q] << 16);
+      y -= __uint_as_float(p[q] & 0xFFFF0000u);
+    }
+  }
+}
+
+// untiled bulk copy global -> shared (16-byte aligned addresses and size)
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
 // mbarrier arrives once all previously issued tcgen05 operations of this thread complete
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");

@@ -1,0 +1,583 @@
+// The weight gradient's last step on the tensor cores (Sec. 2.3, adjoint of the collapse):
+//   dw[co,s,ci,s',k] = sum_{a,b} M_{s,s'}[k][a][b] G[(s,co,a)][(s',ci,b)],  G = sum_split P
+// per shell pair a GEMM [channel pairs] x [(b,a) entries] x [kernel points k < K <= 64],
+// from the FP32 partials P that the weight-gradient GEMM stored transposed (a column
+// (s',ci,b) holds its rows (s,co,a) contiguously).  FP32 operands as three-part BF16
+// splits, six part products, FP32 accumulation over at most one part of the b range
+// (about 250 (b,a) entries, the sums of the parts added in FP32): the error of the FP32 sum
+// it replaces, which is far below that of the voxel sums in G itself.
+//
+// What bounds it: reading P (58 MB per split at 16 -> 64 channels, 232 MB at 64 -> 64).  On
+// the CUDA cores the step was bound by issue instead (64 FMAs per (b,a) entry and pair).
+// Measured, with the sum of the parts and db: 64 -> 64 channels, 2 splits 0.123 ms (4.5 TB/s of
+// P in the main kernel) against 0.353 on the CUDA cores; 16 -> 64 channels, 3 splits 0.053
+// against 0.106.
+//
+// A persistent CTA walks units (shell s, part of the b range, input shell s', tile of up to
+// 128 channel pairs), consecutive units sharing the part's M images in shared memory:
+//   - warp 0 copies, per b and split, the tile's runs of P (one per input channel, c_out n_out
+//     consecutive floats) into a ring with untiled bulk copies;
+//   - 16 converter warps sum the splits (lane = channel pair, so a lane reads its own n_out
+//     floats: an odd stride, no bank conflicts for odd n_out), split the sum into BF16 parts and
+//     store them to TMEM as the MMA's A operand (no shared-memory round trip);
+//   - one thread issues the MMAs (A from TMEM, M images MN-major from shared memory);
+//   - four warps read the accumulator and store the partial sums, lanes along the pairs.
+#include <algorithm>
+#include <vector>
+
+#include "tc_gemm.h"
+#include "tc_ptx.cuh"
+
+namespace delimit {
+
+namespace {
+
+constexpr int kRdN = 64;          // kernel points (MMA N), zero-padded
+constexpr int kRdConvWarps = 16;  // four per TMEM lane quarter
+constexpr int kRdThreads = 32 * (2 + 4 + kRdConvWarps);
+constexpr int kRdMaxKs = 8;       // k-steps of 16 output coefficients per b
+constexpr int kRdRing = 6;        // most ring slots
+constexpr int kRdABufs = 4;       // most A buffers
+constexpr size_t kRdSmemLimit = 226 * 1024;
+constexpr uint32_t kRdDCols = 2 * kRdN;
+
+enum : int {
+  kErrRdRing = 0x5100,
+  kErrRdRingEmpty = 0x5200,
+  kErrRdA = 0x5300,
+  kErrRdAEmpty = 0x5400,
+  kErrRdD = 0x5500,
+  kErrRdDEmpty = 0x5600,
+  kErrRdB = 0x5700,
+  kErrRdDrain = 0x5800
+};
+
+// M_{s,s'} -> three BF16 parts, per (pg, b) an image [part][16 ks rows a][64 kernel points] in
+// the MN-major 128-byte-swizzled operand layout, zero past n_out and K
+__global__ void dw_images_kernel(const __grid_constant__ LscDims d, const float* __restrict__ M,
+                                 uint8_t* __restrict__ img, int npg, int ks) {
+  const int rows = 16 * ks;
+  const int64_t n = (int64_t)npg * d.n_in * rows * kRdN;
+  const int s_of = d.m_stride_sp ? d.s_in : 1;  // resampling-free tables hold one block per shell pair
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int k = (int)(i % kRdN);
+    int64_t r = i / kRdN;
+    const int a = (int)(r % rows);
+    r /= rows;
+    const int b = (int)(r % d.n_in), pg = (int)(r / d.n_in);
+    const int s = pg / s_of, sp = pg - s * s_of;
+    const float x = (k < d.K && a < d.n_out)
+                        ? M[s * d.m_stride_s + sp * d.m_stride_sp + ((int64_t)k * d.n_out + a) * d.n_in + b]
+                        : 0.f;
+    const __nv_bfloat16 x0 = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(x0);
+    const __nv_bfloat16 x1 = __float2bfloat16_rn(r1);
+    const __nv_bfloat16 x2 = __float2bfloat16_rn(r1 - __bfloat162float(x1));
+    uint8_t* base = img + ((int64_t)pg * d.n_in + b) * (3 * rows * 128);
+    const int off = a * 128 + (((k >> 3) ^ (a & 7)) << 4) + (k & 7) * 2;
+    *reinterpret_cast<__nv_bfloat16*>(base + off) = x0;
+    *reinterpret_cast<__nv_bfloat16*>(base + rows * 128 + off) = x1;
+    *reinterpret_cast<__nv_bfloat16*>(base + 2 * rows * 128 + off) = x2;
+  }
+}
+
+}  // namespace
+
+struct RdParams {
+  LscDims d;
+  const float* P;
+  const uint8_t* img;
+  float* dwp;  // [part][k][row of pairs], row = ((s s_in + s') c_in + ci) c_out + co
+  int64_t ldpt, split_stride, part_stride, rows_total;
+  int splits, ks, bpp, nparts;
+  int nseg, co_chunks, ntiles;  // a tile: nseg input channels x all c_out, or one channel x 128 outputs
+  int ring, abufs;
+  uint32_t seg_stride, ring_bytes, img_bytes;  // img_bytes: one b's image
+  int64_t units;
+  int pg_per_pair;
+  int* err;
+};
+
+// one unit of work and its walk: (s, part, s', tile), tile fastest
+struct RdUnit {
+  int s, part, sp, tile;
+  __device__ __forceinline__ void init(const RdParams& p, int64_t u) {
+    s = 0;
+    while (true) {
+      const int64_t n = (int64_t)p.nparts * (p.d.win_hi[s] - p.d.win_lo[s]) * p.ntiles;
+      if (u < n) break;
+      u -= n;
+      ++s;
+    }
+    const int nw = p.d.win_hi[s] - p.d.win_lo[s];
+    tile = (int)(u % p.ntiles);
+    u /= p.ntiles;
+    sp = p.d.win_lo[s] + (int)(u % nw);
+    part = (int)(u / nw);
+  }
+  __device__ __forceinline__ void next(const RdParams& p) {
+    if (++tile < p.ntiles) return;
+    tile = 0;
+    if (++sp < p.d.win_hi[s]) return;
+    if (++part >= p.nparts) {
+      part = 0;
+      do {
+        ++s;
+      } while (s < p.d.s_out && p.d.win_hi[s] <= p.d.win_lo[s]);
+    }
+    if (s < p.d.s_out) sp = p.d.win_lo[s];
+  }
+  // images of this unit's part: equal keys share them
+  __device__ __forceinline__ int key(const RdParams& p) const {
+    const int pg = p.pg_per_pair ? s * p.d.s_in + sp : s;
+    return pg * p.nparts + part;
+  }
+};
+
+__global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __grid_constant__ RdParams p) {
+  using namespace ptx;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const LscDims& d = p.d;
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t ring_off = (uint32_t)p.bpp * p.img_bytes;  // [images of a part][ring slots][barriers]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ring_off + (uint32_t)p.ring * p.ring_bytes);
+  // bars: ring_full[6], ring_empty[6], a_full[4], a_empty[4], d_full[2], d_empty[2], b_full, b_empty, drain
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kRdRing + 2 * kRdABufs + 7);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  auto ring_full = [&](int i) { return smem_u32(bars + i); };
+  auto ring_empty = [&](int i) { return smem_u32(bars + kRdRing + i); };
+  auto a_full = [&](int i) { return smem_u32(bars + 2 * kRdRing + i); };
+  auto a_empty = [&](int i) { return smem_u32(bars + 2 * kRdRing + kRdABufs + i); };
+  auto d_full = [&](int i) { return smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + i); };
+  auto d_empty = [&](int i) { return smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 2 + i); };
+  const uint32_t b_full = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 4);
+  const uint32_t b_empty = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 5);
+  const uint32_t drain_bar = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 6);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kRdRing; ++i) {
+      mbar_init(ring_full(i), 1);
+      mbar_init(ring_empty(i), kRdConvWarps);
+    }
+    for (int i = 0; i < kRdABufs; ++i) {
+      mbar_init(a_full(i), kRdConvWarps);
+      mbar_init(a_empty(i), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(d_full(i), 1);
+      mbar_init(d_empty(i), 4);
+    }
+    mbar_init(b_full, 1);
+    mbar_init(b_empty, 1);
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t a_cols = (uint32_t)(24 * p.ks);  // TMEM columns of one A buffer: 3 parts x 8 per k-step
+  // this CTA's consecutive units
+  const int64_t u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
+  const int cw = d.c_out < 128 ? d.c_out : 128;  // output channels of a full tile row of segments
+
+  if (warp == 0) {
+    // ---- producer: M images when the part changes, then P's runs per (b, split) ----
+    RdUnit un;
+    un.init(p, u0);
+    int key = -1, slot = 0;
+    uint32_t ph = 0, b_ph = 0;
+    uint32_t used = 0;  // ring slots that have been filled
+    int b_loads = 0;
+    bool ok = true;
+    for (int64_t u = u0; u < u1 && ok && !*abort_flag; ++u, un.next(p)) {
+      const int b0 = un.part * p.bpp, nb = min(p.bpp, d.n_in - b0);
+      if (un.key(p) != key) {
+        // the images of the units before are read by MMAs that have completed
+        ok = key < 0 || wait_bounded(b_empty, b_ph, abort_flag, p.err, kErrRdB);
+        if (key >= 0) b_ph ^= 1u;
+        if (!__all_sync(0xffffffffu, ok)) break;
+        key = un.key(p);
+        ++b_loads;
+        if (lane == 0) {
+          const int pg = key / p.nparts;
+          mbar_arrive_expect_tx(b_full, (uint32_t)nb * p.img_bytes);
+          bulk_load(sbase, p.img + ((int64_t)pg * d.n_in + b0) * p.img_bytes, (uint32_t)nb * p.img_bytes, b_full);
+        }
+      }
+      const int co0 = d.c_out < 128 ? 0 : (un.tile % p.co_chunks) * 128;
+      const int ci0 = d.c_out < 128 ? un.tile * p.nseg : un.tile / p.co_chunks;
+      const int len = min(cw, d.c_out - co0) * d.n_out;  // floats of a run
+      const int nsg = min(p.nseg, d.c_in - ci0);
+      const int64_t row = ((int64_t)un.s * d.c_out + co0) * d.n_out;
+      const int mis = (int)(row & 3);  // runs start on 16-byte boundaries; ldpt and split_stride are multiples of 4
+      const uint32_t bytes = (uint32_t)((mis + len + 3) / 4 * 16);
+      for (int b = b0; b < b0 + nb && ok; ++b) {
+        for (int z = 0; z < p.splits; ++z) {
+          ok = wait_bounded(ring_empty(slot), ph ^ 1u, abort_flag, p.err, kErrRdRingEmpty);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive_expect_tx(ring_full(slot), (uint32_t)nsg * bytes);
+          __syncwarp();
+          const uint32_t dst = sbase + ring_off + (uint32_t)slot * p.ring_bytes;
+          for (int g = lane; g < nsg; g += 32)
+            bulk_load(dst + (uint32_t)g * p.seg_stride,
+                      p.P + z * p.split_stride + (((int64_t)un.sp * d.c_in + ci0 + g) * d.n_in + b) * p.ldpt + row - mis,
+                      bytes, ring_full(slot));
+          used |= 1u << slot;
+          if (++slot == p.ring) {
+            slot = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+    }
+    // copies still in flight complete before the CTA may exit: the last fill of every slot used
+    // (slots before `slot` were filled in this pass of the ring, the others in the one before)
+    if (b_loads) wait_drain(b_full, (uint32_t)(b_loads - 1) & 1u, p.err, kErrRdDrain);
+    for (int i = 0; i < p.ring; ++i)
+      if (used >> i & 1u) wait_drain(ring_full(i), i < slot ? ph : ph ^ 1u, p.err, kErrRdDrain);
+  } else if (warp == 1) {
+    if (lane == 0) {
+      RdUnit un;
+      un.init(p, u0);
+      const uint32_t idesc = idesc_bf16(128, kRdN, false, true);
+      const uint32_t part_bytes = (uint32_t)p.ks * 2048u;
+      int key = -1, buf = 0;
+      uint32_t a_ph = 0, b_ph = 0;
+      bool ok = true;
+      for (int64_t u = u0; u < u1 && ok && !*abort_flag; ++u) {
+        const int acc = (int)((u - u0) & 1);
+        const uint32_t d_use = (uint32_t)(((u - u0) >> 1) & 1);
+        const int nb = min(p.bpp, d.n_in - un.part * p.bpp);
+        if (un.key(p) != key) {
+          key = un.key(p);
+          if (!wait_bounded(b_full, b_ph, abort_flag, p.err, kErrRdB)) break;
+          b_ph ^= 1u;
+        }
+        if (!wait_bounded(d_empty(acc), d_use ^ 1u, abort_flag, p.err, kErrRdDEmpty)) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kRdN);
+        for (int b = 0; b < nb; ++b) {
+          if (!wait_bounded(a_full(buf), a_ph, abort_flag, p.err, kErrRdA)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t a_tmem = tmem_base + kRdDCols + (uint32_t)buf * a_cols;
+          const uint32_t b_src = sbase + (uint32_t)b * p.img_bytes;
+          for (int kk = 0; kk < p.ks; ++kk) {
+#pragma unroll
+            for (int pr = 0; pr < 6; ++pr) {  // part products, smallest first
+              constexpr int pa[6] = {2, 1, 0, 1, 0, 0}, pb[6] = {0, 1, 2, 0, 1, 0};
+              const uint64_t bd = umma_desc(b_src + pb[pr] * part_bytes + kk * 2048, part_bytes, 1024, kSwizzle128B);
+              mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(pa[pr] * 8 * p.ks + kk * 8), bd, idesc, (b | kk | pr) != 0);
+            }
+          }
+          mma_commit(a_empty(buf));
+          if (++buf == p.abufs) {
+            buf = 0;
+            a_ph ^= 1u;
+          }
+        }
+        if (!ok) break;
+        mma_commit(d_full(acc));
+        un.next(p);
+        if (u + 1 < u1 && un.key(p) != key) mma_commit(b_empty);
+      }
+      mma_commit(drain_bar);
+      wait_drain(drain_bar, 0, p.err, kErrRdDrain);
+    }
+  } else if (warp < 6) {
+    // ---- epilogue: lane = channel pair of the tile, columns = kernel points ----
+    const int q = warp & 3, r = q * 32 + lane;
+    RdUnit un;
+    un.init(p, u0);
+    for (int64_t u = u0; u < u1; ++u, un.next(p)) {
+      const int acc = (int)((u - u0) & 1);
+      const bool ok = wait_bounded_sleep(d_full(acc), (uint32_t)(((u - u0) >> 1) & 1), abort_flag, p.err, kErrRdD);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      const uint32_t tl = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kRdN);
+      const int co0 = d.c_out < 128 ? 0 : (un.tile % p.co_chunks) * 128;
+      const int ci0 = d.c_out < 128 ? un.tile * p.nseg : un.tile / p.co_chunks;
+      const int g = r / cw, co = co0 + r - g * cw;
+      const bool valid = g < p.nseg && ci0 + g < d.c_in && co < d.c_out;
+      float* out = p.dwp + un.part * p.part_stride +
+                   (((int64_t)un.s * d.s_in + un.sp) * d.c_in + ci0 + g) * d.c_out + co;
+#pragma unroll
+      for (int h = 0; h < kRdN; h += 32) {
+        uint32_t rv[2][16];
+        tmem_ld16_nowait(tl + h, rv[0]);
+        tmem_ld16_nowait(tl + h + 16, rv[1]);
+        tmem_wait_ld();
+        if (valid) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if (h + k < d.K) out[(h + k) * p.rows_total] = __uint_as_float(rv[k >> 4][k & 15]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(d_empty(acc));
+    }
+  } else {
+    // ---- converters: lane = channel pair; warp `sub` of a quarter takes every fourth k-step ----
+    const int q = warp & 3, sub = (warp - 6) >> 2, r = q * 32 + lane;
+    const int g = r / cw, cl = r - g * cw;
+    RdUnit un;
+    un.init(p, u0);
+    int slot = 0, buf = 0;
+    uint32_t ph = 0, a_ph = 0;
+    bool ok = true;
+    for (int64_t u = u0; u < u1 && ok; ++u, un.next(p)) {
+      const int nb = min(p.bpp, d.n_in - un.part * p.bpp);
+      const int co0 = d.c_out < 128 ? 0 : (un.tile % p.co_chunks) * 128;
+      const int ci0 = d.c_out < 128 ? un.tile * p.nseg : un.tile / p.co_chunks;
+      const bool valid = g < p.nseg && ci0 + g < d.c_in && co0 + cl < d.c_out;
+      const int mis = (int)((((int64_t)un.s * d.c_out + co0) * d.n_out) & 3);
+      const uint32_t lane_off = valid ? (uint32_t)g * p.seg_stride + (uint32_t)(mis + cl * d.n_out) * 4u : 0u;
+      for (int b = 0; b < nb && ok; ++b) {
+        const int kk0 = (sub - b * p.ks) & 3;  // this warp's k-steps of this b: kk0, kk0 + 4
+        float v[kRdMaxKs / 4][16];
+#pragma unroll
+        for (int i = 0; i < kRdMaxKs / 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[i][j] = 0.f;
+        for (int z = 0; z < p.splits; ++z) {
+          ok = wait_bounded_sleep(ring_full(slot), ph, abort_flag, p.err, kErrRdRing);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (valid) {
+            const float* src = reinterpret_cast<const float*>(smem + ring_off + (uint32_t)slot * p.ring_bytes + lane_off);
+#pragma unroll
+            for (int i = 0; i < kRdMaxKs / 4; ++i) {
+              const int a0 = 16 * (kk0 + 4 * i);
+              if (a0 + 16 <= d.n_out) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[i][j] += src[a0 + j];
+              } else if (a0 < d.n_out) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (a0 + j < d.n_out) v[i][j] += src[a0 + j];
+              }
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(ring_empty(slot));
+          if (++slot == p.ring) {
+            slot = 0;
+            ph ^= 1u;
+          }
+        }
+        if (!ok) break;
+        ok = wait_bounded_sleep(a_empty(buf), a_ph ^ 1u, abort_flag, p.err, kErrRdAEmpty);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + kRdDCols + (uint32_t)buf * a_cols;
+#pragma unroll
+        for (int i = 0; i < kRdMaxKs / 4; ++i) {
+          const int kk = kk0 + 4 * i;
+          if (kk < p.ks) {
+            uint32_t part[3][8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              uint32_t t3[3];
+              split3x2(v[i][2 * j], v[i][2 * j + 1], t3);
+#pragma unroll
+              for (int t = 0; t < 3; ++t) part[t][j] = t3[t];
+            }
+#pragma unroll
+            for (int t = 0; t < 3; ++t) tmem_st8(at + (uint32_t)(t * 8 * p.ks + kk * 8), part[t]);
+          }
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(a_full(buf));
+        if (++buf == p.abufs) {
+          buf = 0;
+          a_ph ^= 1u;
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// dw = sum of the parts in order (zero outside the window), 32 pairs x K points per block through
+// shared memory ([k][pair] in, [pair][k] out), and db in the blocks after them, one warp per
+// (co, s): db[co,s] = sum_a q[s][a] (row sum of dY's row (s,co,a) over the splits)
+__global__ void __launch_bounds__(256) finish_dw_kernel(const __grid_constant__ RdParams p, float* __restrict__ dw,
+                                                        float* __restrict__ db, const float* __restrict__ qv,
+                                                        int64_t dw_blocks) {
+  __shared__ float t[kRdN][33];
+  const LscDims& d = p.d;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if ((int64_t)blockIdx.x < dw_blocks) {
+    const int64_t r0 = (int64_t)blockIdx.x * 32, row = r0 + lane;
+    auto decode = [&](int64_t r, int& s, int& sp, int& ci, int& co) {
+      co = (int)(r % d.c_out);
+      r /= d.c_out;
+      ci = (int)(r % d.c_in);
+      r /= d.c_in;
+      sp = (int)(r % d.s_in);
+      s = (int)(r / d.s_in);
+    };
+    int s, sp, ci, co;
+    decode(row < p.rows_total ? row : 0, s, sp, ci, co);
+    const bool in = row < p.rows_total && sp >= d.win_lo[s] && sp < d.win_hi[s];
+    for (int k = warp; k < d.K; k += 8) {
+      float a = 0.f;
+      if (in)
+        for (int z = 0; z < p.nparts; ++z) a += p.dwp[z * p.part_stride + k * p.rows_total + row];
+      t[k][lane] = a;
+    }
+    __syncthreads();
+    for (int i = warp; i < 32; i += 8) {
+      if (r0 + i >= p.rows_total) break;
+      decode(r0 + i, s, sp, ci, co);
+      float* out = dw + ((((int64_t)co * d.s_out + s) * d.c_in + ci) * d.s_in + sp) * d.K;
+      for (int k = lane; k < d.K; k += 32) out[k] = t[k][i];
+    }
+  } else {
+    const int64_t i = ((int64_t)blockIdx.x - dw_blocks) * 8 + warp;
+    if (i >= (int64_t)d.c_out * d.s_out) return;
+    const int co = (int)(i / d.s_out), s = (int)(i % d.s_out);
+    const int64_t row0 = ((int64_t)s * d.c_out + co) * d.n_out;
+    float acc = 0.f;
+    for (int aa = lane; aa < d.n_out; aa += 32) {
+      float r = 0.f;
+      for (int z = 0; z < p.splits; ++z) r += p.P[z * p.split_stride + d.rows_in * p.ldpt + row0 + aa];
+      acc = fmaf(qv[s * d.n_out + aa], r, acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) db[co * d.s_out + s] = acc;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+namespace {
+
+int rd_bpp(int n_in, int n_out) {
+  // as many parts of the b range as the CUDA-core reduction has parts of 256 (a,b) entries
+  const int parts = (n_in * n_out + 255) / 256;
+  return (n_in + parts - 1) / parts;
+}
+
+// shared memory beside the ring: the part's images, alignment and barriers
+size_t rd_fixed(int n_in, int n_out) {
+  const int ks = (n_out + 15) / 16;
+  return 1024 + (size_t)rd_bpp(n_in, n_out) * 3 * ks * 2048 + (2 * kRdRing + 2 * kRdABufs + 7) * 8 + 64;
+}
+
+}  // namespace
+
+cudaError_t reduce_dw_tables_create(const LscDims& dt, const float* d_M, ReduceDwTables& t, std::string& err) {
+  t = ReduceDwTables();
+  const int ks = (dt.n_out + 15) / 16;
+  // more kernel points, coefficients or images than the kernel holds: the CUDA-core reduction
+  if (dt.K > kRdN || ks > kRdMaxKs || rd_fixed(dt.n_in, dt.n_out) + 2 * 128 * (size_t)(4 * dt.n_out + 32) > kRdSmemLimit)
+    return cudaSuccess;
+  t.npg = dt.m_stride_sp ? dt.s_out * dt.s_in : dt.s_out;
+  const size_t bytes = (size_t)t.npg * dt.n_in * 3 * ks * 2048;
+  cudaError_t e = cudaMalloc(&t.d_img, bytes);
+  if (e == cudaSuccess) {
+    dw_images_kernel<<<152 * 4, 256>>>(dt, d_M, static_cast<uint8_t*>(t.d_img), t.npg, ks);
+    count_launch();
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  }
+  if (e != cudaSuccess) {
+    err = cudaGetErrorString(e);
+    if (t.d_img) cudaFree(t.d_img);
+    t = ReduceDwTables();
+    return e;
+  }
+  t.ok = true;
+  return cudaSuccess;
+}
+
+void reduce_dw_tables_destroy(ReduceDwTables& t) {
+  if (t.d_img) cudaFree(t.d_img);
+  t = ReduceDwTables();
+}
+
+bool tc_reduce_dw_supported(const ReduceDwTables& t) {
+  if (!t.ok || !tc_enabled()) return false;
+  int dev = 0, major = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+  return major == 10;
+}
+
+cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float* P, int64_t ldpt, int64_t split_stride,
+                         int splits, const float* q, float* dw, float* db, float* scratch, int* err, cudaStream_t st) {
+  TraceScope trace("lsc_reduce_dw", st);
+  RdParams p;
+  memset(&p, 0, sizeof p);
+  p.d = d;
+  p.P = P;
+  p.img = static_cast<const uint8_t*>(t.d_img);
+  p.dwp = scratch;
+  p.ldpt = ldpt;
+  p.split_stride = split_stride;
+  p.splits = splits;
+  p.ks = (d.n_out + 15) / 16;
+  p.bpp = rd_bpp(d.n_in, d.n_out);
+  p.nparts = (d.n_in + p.bpp - 1) / p.bpp;
+  p.rows_total = (int64_t)d.s_out * d.s_in * d.c_in * d.c_out;
+  p.part_stride = p.rows_total * d.K;
+  p.nseg = d.c_out < 128 ? 128 / d.c_out : 1;
+  p.co_chunks = d.c_out < 128 ? 1 : (d.c_out + 127) / 128;
+  p.ntiles = d.c_out < 128 ? (d.c_in + p.nseg - 1) / p.nseg : d.c_in * p.co_chunks;
+  p.seg_stride = (uint32_t)((std::min(d.c_out, 128) * d.n_out + 3 + 3) / 4 * 16);
+  p.ring_bytes = (uint32_t)(p.nseg * p.seg_stride);
+  p.img_bytes = (uint32_t)(3 * p.ks * 2048);
+  p.pg_per_pair = d.m_stride_sp ? 1 : 0;
+  p.err = err;
+  for (int s = 0; s < d.s_out; ++s) p.units += (int64_t)p.nparts * std::max(0, d.win_hi[s] - d.win_lo[s]) * p.ntiles;
+  cudaError_t e;
+  if (dw && p.units > 0) {
+    const size_t fixed = rd_fixed(d.n_in, d.n_out);
+    p.ring = (int)std::min<size_t>(kRdRing, (kRdSmemLimit - fixed) / p.ring_bytes);
+    if (p.ring < 2) return cudaErrorInvalidValue;
+    p.abufs = std::min(kRdABufs, (int)((512 - kRdDCols) / (24 * p.ks)));
+    // at least 120 KiB so that two CTAs never share an SM (each holds 512 TMEM columns)
+    const size_t smem = std::max<size_t>(120 * 1024, fixed + (size_t)p.ring * p.ring_bytes);
+    e = cudaFuncSetAttribute(reduce_dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const unsigned grid = (unsigned)std::min<int64_t>(p.units, std::max(1, sms));
+    reduce_dw_tc_kernel<<<grid, kRdThreads, smem, st>>>(p);
+    count_launch();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t dw_blocks = dw ? (p.rows_total + 31) / 32 : 0;
+  const int64_t db_blocks = db ? ((int64_t)d.c_out * d.s_out + 7) / 8 : 0;
+  if (dw_blocks + db_blocks == 0) return cudaSuccess;
+  finish_dw_kernel<<<(unsigned)(dw_blocks + db_blocks), 256, 0, st>>>(p, dw, db, q, dw_blocks);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace delimit

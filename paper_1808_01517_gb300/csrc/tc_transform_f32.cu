@@ -78,21 +78,6 @@ struct Tf32Params {
 __constant__ int8_t kProdA[6] = {2, 1, 0, 1, 0, 0};
 __constant__ int8_t kProdB[6] = {0, 1, 2, 0, 1, 0};
 
-// (x, y) -> BF16 parts packed in pairs: x = x0 + x1 + x2 and y likewise, each part the
-// round-to-nearest BF16 of what the earlier ones leave (the differences are exact in FP32);
-// p[q] holds part q of x in its low and of y in its high half
-__device__ __forceinline__ void split3x2(float x, float y, uint32_t (&p)[3]) {
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    p[q] = *reinterpret_cast<const uint32_t*>(&h);
-    if (q < 2) {
-      x -= __uint_as_float(p[q] << 16);
-      y -= __uint_as_float(p[q] & 0xFFFF0000u);
-    }
-  }
-}
-
 // (tile, chunk) of a CTA's work in 32-bit steps: tile t = local + k * ncta = c * m_tiles + mt
 struct Walk {
   int k, ch, c, mt;
