@@ -744,9 +744,7 @@ cudaError_t build_operator(const LscDims& d, const delimit_lsc_geometry* g, cons
                            cudaStream_t cs) {
   const bool wt = needs_wt(d, tc, act_t);
   if (tc && act_t == DELIMIT_BF16 && !wt && tc_build_w_supported(d, g->bw)) {
-    cudaError_t e = tc_build_w(d, g->bw, w, W, g->err_word, cs);
-    if (e != cudaSuccess || !bias) return e;
-    return launch_build_bias(d, b, g->d_q, bias, cs);
+    return tc_build_w(d, g->bw, w, b, g->d_q, W, bias, g->err_word, cs);
   }
   cudaError_t e = launch_build_w(d, w, b, g->d_M, g->d_q, W, wt ? Wt : nullptr, bias, int(act_t), cs);
   if (e != cudaSuccess || !(tc && act_t == DELIMIT_F32)) return e;

@@ -1,29 +1,32 @@
 // The collapsed LSC operator on the tensor cores (Sec. 2.3, the exact collapse of the
 // resample / product / projection steps into one matrix per shell pair):
 //   W[(s,co,a)][(s',ci,b)] = sum_k w[co,s,ci,s',k] M_{s,s'}[k][a][b]
-// per shell pair a GEMM [channel pairs p = co c_in + ci] x [kernel points k < K] x
-// [(a,b) entries], with K <= 64 (padded with zeros to 64).  FP32 operands on the BF16
-// tensor cores as three-part splits (x = x0 + x1 + x2 to 2^-27 |x|, the six part
-// products down to 2^-18 of the leading one, FP32 accumulation in TMEM): FP32-level
-// accuracy before the result is rounded to BF16 (the same rounding point as the
-// CUDA-core build).  The parts of M are made once per geometry (M is fixed).
+// per shell pair a GEMM [channel pairs (co, ci)] x [kernel points k < K <= 64] x [(a,b)
+// entries].  FP32 operands on the BF16 tensor cores as three-part splits (x = x0 + x1 + x2
+// to 2^-27 |x|, the six part products down to 2^-18 of the leading one, FP32 accumulation in
+// TMEM): FP32-level accuracy before the result is rounded to BF16 (the same rounding point as
+// the CUDA-core build).  The parts of M are made once per geometry (M is fixed).
 //
-// One CTA per (shell pair, 128 channel pairs, 256 (a,b) entries), c_in dividing 128 so
-// that a tile holds whole output channels:
-//   - the CTA splits its 128 x 64 slice of w into three BF16 parts, written straight into
-//     the K-major 128-byte-swizzled operand layout; one thread loads the three M parts
-//     (MN-major, four 64-entry atoms x 64 k each) by TMA, issues the 24 MMAs (M = 128,
-//     N = 256, K = 16) and commits;
-//   - 32 warps read the accumulator (eight per TMEM lane quarter), round to BF16 and
-//     scatter it into a staging tile in W's own order [co][a][ci][b] (in the freed
-//     operand space), so that every row run of W the tile covers, (s, co, a) with the
-//     tile's channels ci and their b entries, is contiguous there;
-//   - the warps copy the runs out, 16 bytes per lane where the run is whole and aligned.
-// Shell pairs outside the window write zeros.  Every wait is bounded.
-#include <cudaTypedefs.h>
-
+// What bounds it: the MMAs (144 of them per 128 pairs and four rows), close behind them writing
+// W (149 MB at 64 -> 64 channels, 29 MB at 16 -> 64).  One tile per CTA took 20 us, its loads,
+// MMAs, TMEM reads and stores one after the other; a persistent CTA that overlaps them, with
+// tiles of whole rows a so that every run of W leaves in one copy, measured 0.304 -> 0.083 ms
+// (64 -> 64 channels) and 0.058 -> 0.030 (16 -> 64).
+//
+// A tile is (output shell s, two halves of 128 / n_in rows a with all their b entries, input
+// shell s', 128 / c_in output channels with all their input channels).  A CTA walks consecutive
+// tiles that share the M image of (s, rows) in shared memory:
+//   - four loader warps copy the tile's w (4-byte cp.async: w needs no alignment) into a ring,
+//     and the M image when it changes;
+//   - 8 converter warps split w into BF16 parts and store them to TMEM as the MMA's A operand;
+//   - one thread issues the MMAs (6 part products, A from TMEM, M = 128 pairs, N = a half's
+//     entries), a half's while the other's accumulator is read;
+//   - 8 epilogue warps read the accumulator, round to BF16 and write a staging tile in W's own
+//     order [co][a][ci][b];
+//   - one warp copies the staging tile's rows, contiguous in W, out with bulk copies, and at the
+//     end writes zeros outside the shell window.
+// Every wait is bounded.
 #include <algorithm>
-#include <mutex>
 
 #include "tc_gemm.h"
 #include "tc_ptx.cuh"
@@ -32,220 +35,407 @@ namespace delimit {
 
 namespace {
 
-constexpr int kBwTP = 128;                              // channel pairs per tile (MMA M)
-constexpr int kBwTN = 256;                              // (a,b) entries per tile (MMA N)
-constexpr int kBwK = 64;                                // kernel points, zero-padded
-constexpr uint32_t kBwABytes = kBwTP * kBwK * 2;         // one w part tile: 16 KiB
-constexpr uint32_t kBwBBytes = kBwTN * kBwK * 2;         // one M part tile: 4 atoms x 8 KiB
-constexpr uint32_t kBwOpBytes = 3 * (kBwABytes + kBwBBytes);  // 144 KiB
-constexpr int kBwThreads = 1024;
-constexpr int kErrBwLoad = 0x4A00, kErrBwMma = 0x4B00;
+constexpr int kBwK = 64;                        // kernel points, zero-padded
+constexpr int kBwMaxN = 256;                    // TMEM columns of the accumulators
+constexpr int kBwAtomBytes = kBwK * 128;        // one 64-entry atom of an M part: [64 k][64 entries]
+constexpr int kBwLoadWarps = 4, kBwEpiWarps = 8, kBwConvWarps = 8;
+constexpr int kBwEpi0 = kBwLoadWarps + 2, kBwConv0 = kBwEpi0 + kBwEpiWarps;  // first warp of a role
+constexpr int kBwThreads = 32 * (kBwConv0 + kBwConvWarps);
+constexpr size_t kBwSmemLimit = 226 * 1024;
+constexpr uint32_t kBwACols = 96;               // TMEM columns of an A buffer: 3 parts x 32
 
-// the six part products, largest first: term t multiplies part pa(t) of w with part pb(t) of M
-__host__ __device__ constexpr int bw_part_a(int t) { return t == 2 || t == 3 ? 1 : (t == 5 ? 2 : 0); }
-__host__ __device__ constexpr int bw_part_b(int t) { return t == 1 || t == 3 ? 1 : (t == 4 ? 2 : 0); }
+enum : int {
+  kErrBwW = 0x4100,
+  kErrBwWEmpty = 0x4200,
+  kErrBwA = 0x4300,
+  kErrBwAEmpty = 0x4400,
+  kErrBwD = 0x4500,
+  kErrBwDEmpty = 0x4600,
+  kErrBwStg = 0x4700,
+  kErrBwStgFree = 0x4800,
+  kErrBwM = 0x4900,
+  kErrBwDrain = 0x4A00
+};
 
-// two BF16 values' bits in one word, lo in the low half
-__device__ __forceinline__ uint32_t bf16_bits2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
+// halves of a tile (an accumulator and a staging buffer each), rows a of a half and of a tile,
+// tiles of a shell's n_out rows, 64-entry atoms of a half's M image
+__host__ __device__ constexpr int bw_halves(int n_in) { return n_in <= 128 ? 2 : 1; }
+__host__ __device__ constexpr int bw_hrows(int n_in) { return n_in <= 128 ? 128 / n_in : 1; }
+__host__ __device__ constexpr int bw_rows(int n_in) { return bw_halves(n_in) * bw_hrows(n_in); }
+__host__ __device__ constexpr int bw_tiles(int n_in, int n_out) { return (n_out + bw_rows(n_in) - 1) / bw_rows(n_in); }
+__host__ __device__ constexpr int bw_atoms(int n_in) { return (bw_hrows(n_in) * n_in + 63) / 64; }
 
-// (a,b) rows a tile of 256 entries touches, at most
-__host__ __device__ constexpr int bw_max_rows(int n_in) { return (kBwTN - 1) / n_in + 2; }
-
-// M_{s,s'} -> its three BF16 parts, per shell pair pg a [64][ldm] MN-major block (kernel
-// point k, entry ab; zero past K points and nab entries).  Scalar loads: M's rows of
-// n_out n_in floats need not be 16-byte aligned.
+// M_{s,s'} -> its three BF16 parts, per (shell or shell pair, tile of rows) an operand image
+// [part][half][atom][64 k][64 entries], MN-major with the 128-byte swizzle, entry
+// e = (a - a0) n_in + b of a half, zero past its rows and K
 __global__ void split_m_kernel(const __grid_constant__ LscDims d, const float* __restrict__ M,
-                               __nv_bfloat16* __restrict__ mp, int ldm, int npg) {
-  const int64_t n = (int64_t)npg * kBwK * ldm;
-  const int nab = d.n_out * d.n_in;
+                               uint8_t* __restrict__ img, int npg) {
+  const int hr = bw_hrows(d.n_in), nh = bw_halves(d.n_in), nt = bw_tiles(d.n_in, d.n_out), ha = bw_atoms(d.n_in);
+  const int atoms = nh * ha;
+  const int64_t n = (int64_t)npg * nt * atoms * kBwK * 64;
+  const int s_of = d.m_stride_sp ? d.s_in : 1;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int ab = (int)(i % ldm);
-    const int64_t r = i / ldm;
-    const int k = (int)(r % kBwK), pg = (int)(r / kBwK);
-    const int s = pg / d.s_in, sp = pg - s * d.s_in;
-    const float x = (k < d.K && ab < nab) ? M[s * d.m_stride_s + sp * d.m_stride_sp + (int64_t)k * nab + ab] : 0.f;
+    const int c = (int)(i % 64), k = (int)(i / 64 % kBwK);
+    int64_t r = i / (64 * kBwK);
+    const int at = (int)(r % atoms);
+    r /= atoms;
+    const int t = (int)(r % nt), pg = (int)(r / nt), s = pg / s_of, sp = pg - s * s_of;
+    const int hf = at / ha, e = (at - hf * ha) * 64 + c, al = e / d.n_in, b = e - al * d.n_in, a = (t * nh + hf) * hr + al;
+    const float x = (k < d.K && al < hr && a < d.n_out)
+                        ? M[s * d.m_stride_s + sp * d.m_stride_sp + ((int64_t)k * d.n_out + a) * d.n_in + b]
+                        : 0.f;
     const __nv_bfloat16 x0 = __float2bfloat16_rn(x);
     const float r1 = x - __bfloat162float(x0);
     const __nv_bfloat16 x1 = __float2bfloat16_rn(r1);
-    mp[i] = x0;
-    mp[n + i] = x1;
-    mp[2 * n + i] = __float2bfloat16_rn(r1 - __bfloat162float(x1));
+    uint8_t* base = img + ((int64_t)pg * nt + t) * (3 * atoms * kBwAtomBytes) + at * kBwAtomBytes + k * 128 +
+                    (((c >> 3) ^ (k & 7)) << 4) + (c & 7) * 2;
+    *reinterpret_cast<__nv_bfloat16*>(base) = x0;
+    *reinterpret_cast<__nv_bfloat16*>(base + atoms * kBwAtomBytes) = x1;
+    *reinterpret_cast<__nv_bfloat16*>(base + 2 * atoms * kBwAtomBytes) = __float2bfloat16_rn(r1 - __bfloat162float(x1));
   }
 }
 
 }  // namespace
 
-struct BwMaps {
-  CUtensorMap b;  // M parts: 2-D {ldm entries, 3 npg 64 rows}, box {64, 64}
+struct BwParams {
+  LscDims d;
+  const float* w;
+  const uint8_t* img;
+  const float* b;    // bias and q: the bias vector is made here too (bias null: not wanted)
+  const float* q;
+  float* bias;
+  __nv_bfloat16* W;
+  int64_t units;
+  int nh, hr, nt, atoms, cpt, nptiles, ring, wld;  // cpt: output channels per tile; wld: odd row length of w in the ring
+  int pg_per_pair;
+  uint32_t img_bytes, w_bytes, stg_bytes;  // stg_bytes: one half's staging buffer
+  int* err;
 };
 
-__global__ void __launch_bounds__(kBwThreads, 1)
-    build_w_tc_kernel(const __grid_constant__ BwMaps maps, const __grid_constant__ LscDims d,
-                      const float* __restrict__ w, __nv_bfloat16* __restrict__ W, int vec, int* err) {
+// one tile and its walk: (s, t, s', ptile), ptile fastest
+struct BwUnit {
+  int s, t, sp, pt;
+  __device__ __forceinline__ void init(const BwParams& p, int64_t u) {
+    s = 0;
+    while (true) {
+      const int64_t n = (int64_t)p.nt * (p.d.win_hi[s] - p.d.win_lo[s]) * p.nptiles;
+      if (u < n) break;
+      u -= n;
+      ++s;
+    }
+    const int nw = p.d.win_hi[s] - p.d.win_lo[s];
+    pt = (int)(u % p.nptiles);
+    u /= p.nptiles;
+    sp = p.d.win_lo[s] + (int)(u % nw);
+    t = (int)(u / nw);
+  }
+  __device__ __forceinline__ void next(const BwParams& p) {
+    if (++pt < p.nptiles) return;
+    pt = 0;
+    if (++sp < p.d.win_hi[s]) return;
+    if (++t >= p.nt) {
+      t = 0;
+      do {
+        ++s;
+      } while (s < p.d.s_out && p.d.win_hi[s] <= p.d.win_lo[s]);
+    }
+    if (s < p.d.s_out) sp = p.d.win_lo[s];
+  }
+  __device__ __forceinline__ int key(const BwParams& p) const {
+    return (p.pg_per_pair ? s * p.d.s_in + sp : s) * p.nt + t;
+  }
+};
+
+__global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_constant__ BwParams p) {
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const LscDims& d = p.d;
   const uint32_t sbase = smem_u32(smem);
-  const uint32_t a_base = sbase, b_base = sbase + 3 * kBwABytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBwOpBytes);  // full, done
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+  // [M image][staging buffers][w ring][barriers]
+  const uint32_t stg_off = p.img_bytes, w_off = stg_off + (uint32_t)p.nh * p.stg_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + w_off + (uint32_t)p.ring * p.w_bytes);
+  // bars, two of each: w_full, w_empty, a_full, a_empty, d_full, d_empty, stg_full, stg_free; m_full, m_empty, drain
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const uint32_t full_bar = smem_u32(bars), done_bar = smem_u32(bars + 1);
-  __nv_bfloat16* stg = reinterpret_cast<__nv_bfloat16*>(smem);  // [nco][na][c_in][n_in] after the MMAs
-  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  const int pg = blockIdx.z, s = pg / d.s_in, sp = pg - s * d.s_in;
-  const bool in_win = sp >= d.win_lo[s] && sp < d.win_hi[s];
-  const int nab = d.n_out * d.n_in, npairs = d.c_out * d.c_in;
-  const int p0 = blockIdx.y * kBwTP, np = min(kBwTP, npairs - p0);
-  const int ab0 = blockIdx.x * kBwTN, nabc = min(kBwTN, nab - ab0);
-  const int npg = d.s_out * d.s_in;
-  // c_in divides 128: the tile holds channels co_lo .. co_lo + nco - 1 whole
-  const int co_lo = p0 / d.c_in, nco = np / d.c_in;
-  const int a_lo = ab0 / d.n_in, na = (ab0 + nabc - 1) / d.n_in - a_lo + 1;
-  const int rowlen = d.c_in * d.n_in;
-  bool ok = true;
-  if (in_win) {
-    if (tid == 0) {
-      mbar_init(full_bar, 1);
-      mbar_init(done_bar, 1);
-      *abort_flag = 0;
-      fence_mbar_init();
-      // the three parts of M (kernel points 0 .. 63 of entries ab0 .., four 64-entry atoms
-      // each), in flight while the threads split w
-      mbar_arrive_expect_tx(full_bar, 3 * kBwBBytes);
-      for (int q = 0; q < 3; ++q)
-        for (int at = 0; at < kBwTN / 64; ++at)
-          tma_load_2d(&maps.b, full_bar, b_base + q * kBwBBytes + at * (kBwK * 128), ab0 + 64 * at,
-                      (q * npg + pg) * kBwK);
+  auto w_full = [&](int i) { return smem_u32(bars + i); };
+  auto w_empty = [&](int i) { return smem_u32(bars + 2 + i); };
+  auto a_full = [&](int i) { return smem_u32(bars + 4 + i); };
+  auto a_empty = [&](int i) { return smem_u32(bars + 6 + i); };
+  auto d_full = [&](int i) { return smem_u32(bars + 8 + i); };
+  auto d_empty = [&](int i) { return smem_u32(bars + 10 + i); };
+  auto stg_full = [&](int i) { return smem_u32(bars + 12 + i); };
+  auto stg_free = [&](int i) { return smem_u32(bars + 14 + i); };
+  const uint32_t m_full = smem_u32(bars + 16), m_empty = smem_u32(bars + 17), drain_bar = smem_u32(bars + 18);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(w_full(i), 32 * kBwLoadWarps);
+      mbar_init(w_empty(i), kBwConvWarps);
+      mbar_init(a_full(i), kBwConvWarps);
+      mbar_init(a_empty(i), 1);
+      mbar_init(d_full(i), 1);
+      mbar_init(d_empty(i), kBwEpiWarps);
+      mbar_init(stg_full(i), kBwEpiWarps);
+      mbar_init(stg_free(i), 1);
     }
-    if (warp == 0) {
-      tmem_alloc(smem_u32(tmem_slot), kBwTN);
-      tmem_relinquish();
-    }
-    // the three parts of w: row r = pair p0 + r, 16-byte chunk c = kernel points 8c .. 8c + 7,
-    // stored at r * 128 + ((c ^ r % 8) << 4) of each part (K-major, 128-byte swizzle)
-#pragma unroll
-    for (int e = 0; e < kBwTP * 8 / kBwThreads; ++e) {
-      const int i = tid + kBwThreads * e, r = i >> 3, c = i & 7, p = p0 + r;
-      float x[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = 0.f;
-      if (p < npairs) {
-        const int co = p / d.c_in, ci = p - co * d.c_in;
-        const float* wr = w + ((((int64_t)co * d.s_out + s) * d.c_in + ci) * d.s_in + sp) * d.K;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (8 * c + j < d.K) x[j] = __ldg(wr + 8 * c + j);
-      }
-      uint32_t q0[4], q1[4], q2[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float lo = x[2 * j], hi = x[2 * j + 1];
-        const __nv_bfloat16 l0 = __float2bfloat16_rn(lo), h0 = __float2bfloat16_rn(hi);
-        lo -= __bfloat162float(l0);
-        hi -= __bfloat162float(h0);
-        const __nv_bfloat16 l1 = __float2bfloat16_rn(lo), h1 = __float2bfloat16_rn(hi);
-        lo -= __bfloat162float(l1);
-        hi -= __bfloat162float(h1);
-        q0[j] = bf16_bits2(l0, h0);
-        q1[j] = bf16_bits2(l1, h1);
-        q2[j] = bf16_bits2(__float2bfloat16_rn(lo), __float2bfloat16_rn(hi));
-      }
-      const uint32_t off = (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4));
-      *reinterpret_cast<uint4*>(smem + off) = make_uint4(q0[0], q0[1], q0[2], q0[3]);
-      *reinterpret_cast<uint4*>(smem + kBwABytes + off) = make_uint4(q1[0], q1[1], q1[2], q1[3]);
-      *reinterpret_cast<uint4*>(smem + 2 * kBwABytes + off) = make_uint4(q2[0], q2[1], q2[2], q2[3]);
-    }
-    fence_proxy_async_smem();  // the w parts, written by the threads, before the MMAs read them
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    if (tid == 0) {
-      if (wait_bounded(full_bar, 0, abort_flag, err, kErrBwLoad)) {
-        tc_fence_after();
-        // A K-major (rows of 64 k, 8-row groups 1024 B apart, 16 k = 32 B per MMA); B MN-major
-        // (64-entry atoms 8 KiB apart, 8-k groups 1024 B apart, 16 k = 2048 B per MMA)
-        constexpr uint32_t idesc = idesc_bf16(kBwTP, kBwTN, false, true);
-        bool first = true;
-        for (int ti = 0; ti < 6; ++ti) {
-          const int t = 5 - ti;  // smallest part products first
-          const uint32_t asrc = a_base + bw_part_a(t) * kBwABytes, bsrc = b_base + bw_part_b(t) * kBwBBytes;
-#pragma unroll
-          for (int k = 0; k < kBwK / 16; ++k) {
-            const uint64_t ad = umma_desc(asrc + k * 32, 16, 1024, kSwizzle128B);
-            const uint64_t bd = umma_desc(bsrc + k * 2048, kBwK * 128, 1024, kSwizzle128B);
-            mma_bf16(tmem_base, ad, bd, idesc, !first);
-            first = false;
-          }
-        }
-        mma_commit(done_bar);
-      }
-    }
-    __syncwarp();
-    ok = wait_bounded(done_bar, 0, abort_flag, err, kErrBwMma);
-    tc_fence_after();
-    // accumulator -> BF16 -> staging in W's order: warp w reads TMEM lanes 32 (w % 4) ..
-    // (pairs) and kCols columns from kCols (w / 4) in 16-column loads
-    if (__all_sync(0xffffffffu, ok)) {
-      constexpr int kCols = kBwTN / (kBwThreads / 128);  // columns per warp
-      const int quarter = warp & 3, cq = warp >> 2, prow = 32 * quarter + lane;
-      const bool pv = prow < np;
-      const int co_l = prow / d.c_in, ci = prow - co_l * d.c_in;
-      const uint32_t tl = tmem_base + ((uint32_t)(32 * quarter) << 16);
-      __nv_bfloat16* srow = stg + ((int64_t)co_l * na * d.c_in + ci) * d.n_in;  // + (a - a_lo) rowlen + b
-#pragma unroll 1
-      for (int c = 0; c < kCols; c += 16) {
-        const int col = kCols * cq + c;
-        uint32_t r[16];
-        tmem_ld16_nowait(tl + (uint32_t)col, r);
-        tmem_wait_ld();
-        const int ab = ab0 + col;
-        int a = ab / d.n_in, b = ab - a * d.n_in;
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) {
-          if (pv && col + jj < nabc) srow[(a - a_lo) * rowlen + b] = __float2bfloat16_rn(__uint_as_float(r[jj]));
-          if (++b == d.n_in) {
-            b = 0;
-            ++a;
-          }
-        }
-      }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-      tc_fence_after();
-      tmem_dealloc(tmem_base, kBwTN);
+    mbar_init(m_full, 1);
+    mbar_init(m_empty, 1);
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == kBwLoadWarps) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  if (p.bias) {  // bias_vec[(s,co,a)] = b[co,s] q[s][a]
+    for (int64_t r = (int64_t)blockIdx.x * kBwThreads + threadIdx.x; r < d.rows_out; r += (int64_t)gridDim.x * kBwThreads) {
+      const int per_out = d.c_out * d.n_out;
+      const int s = (int)(r / per_out), co = (int)((r / d.n_out) % d.c_out), aa = (int)(r % d.n_out);
+      p.bias[r] = p.b ? p.b[co * d.s_out + s] * p.q[s * d.n_out + aa] : 0.f;
     }
   }
-  // copy-out: run (co, a) of W's row (s, co, a), columns s' in_blk + (ci, b), from staging
-  // row (co - co_lo, a - a_lo); whole runs in 16-byte chunks when vec, partial ones (the
-  // tile's first and last a) entry by entry
-  const bool have = in_win && ok;
-  for (int r = warp; r < nco * na; r += kBwThreads / 32) {
-    const int co_l = r / na, a_l = r - co_l * na, co = co_lo + co_l, aa = a_lo + a_l;
-    const int b0 = max(0, ab0 - aa * d.n_in), b1 = min(d.n_in, ab0 + nabc - aa * d.n_in);
-    __nv_bfloat16* dst = W + (((int64_t)s * d.c_out + co) * d.n_out + aa) * d.ldW + (int64_t)sp * d.in_blk;
-    const __nv_bfloat16* src = stg + (int64_t)r * rowlen;
-    if (b0 == 0 && b1 == d.n_in) {
-      if (vec) {
-        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-        for (int j = lane; j < rowlen / 8; j += 32)
-          reinterpret_cast<uint4*>(dst)[j] = have ? reinterpret_cast<const uint4*>(src)[j] : z;
-      } else {
-        for (int j = lane; j < rowlen; j += 32) dst[j] = have ? src[j] : __float2bfloat16_rn(0.f);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const int64_t u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
+  const int ksteps = (d.K + 15) / 16;
+  const int rowlen = d.c_in * d.n_in;
+
+  if (warp < kBwLoadWarps) {
+    // ---- loaders: 32 of the tile's 128 pairs each; the first loads the M image too ----
+    BwUnit un;
+    un.init(p, u0);
+    int key = -1, slot = 0, m_loads = 0;
+    uint32_t ph = 0;
+    for (int64_t u = u0; u < u1 && !*abort_flag; ++u, un.next(p)) {
+      bool ok = wait_bounded(w_empty(slot), ph ^ 1u, abort_flag, p.err, kErrBwWEmpty);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (warp == 0 && un.key(p) != key) {
+        // the M image of the tiles before is read by MMAs that have completed
+        ok = m_loads == 0 || wait_bounded(m_empty, (uint32_t)(m_loads - 1) & 1u, abort_flag, p.err, kErrBwM);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        key = un.key(p);
+        ++m_loads;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(m_full, p.img_bytes);
+          bulk_load(sbase, p.img + (int64_t)key * p.img_bytes, p.img_bytes, m_full);
+        }
       }
-    } else {
-      int bj = lane % d.n_in;
-      for (int j = lane; j < rowlen; j += 32) {
-        if (bj >= b0 && bj < b1) dst[j] = have ? src[j] : __float2bfloat16_rn(0.f);
-        bj += 32;
-        while (bj >= d.n_in) bj -= d.n_in;
+      // w rows of the tile's pairs r = (co - co0) c_in + ci, K floats each, at an odd stride
+      const int co0 = un.pt * p.cpt, np = min(p.cpt, d.c_out - co0) * d.c_in;
+      const uint32_t dst0 = sbase + w_off + (uint32_t)slot * p.w_bytes;
+      const int64_t ci_stride = (int64_t)d.s_in * d.K, co_jump = (int64_t)d.s_out * d.c_in * ci_stride;
+      const int r0 = 32 * warp;
+      int ci = r0 % d.c_in;
+      const float* src = p.w + ((((int64_t)(co0 + r0 / d.c_in) * d.s_out + un.s) * d.c_in) * d.s_in + un.sp) * d.K;
+      const float* row = src + ci * ci_stride;
+      for (int r = r0; r < min(np, r0 + 32); ++r) {
+        const uint32_t dst = dst0 + (uint32_t)(r * p.wld + lane) * 4u;
+        if (lane < d.K) cp_async4(dst, row + lane);
+        if (lane + 32 < d.K) cp_async4(dst + 128, row + lane + 32);
+        row += ci_stride;
+        if (++ci == d.c_in) {
+          ci = 0;
+          src += co_jump;
+          row = src;
+        }
+      }
+      cp_async_mbar_arrive(w_full(slot));
+      if (++slot == p.ring) {
+        slot = 0;
+        ph ^= 1u;
       }
     }
+    // copies still in flight complete before the CTA may exit
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (m_loads) wait_drain(m_full, (uint32_t)(m_loads - 1) & 1u, p.err, kErrBwDrain);
+  } else if (warp == kBwLoadWarps) {
+    if (lane == 0) {
+      BwUnit un;
+      un.init(p, u0);
+      int key = -1, m_loads = 0, i = 0;
+      for (int64_t u = u0; u < u1 && !*abort_flag; ++u, ++i) {
+        const int buf = i & 1;
+        if (un.key(p) != key) {
+          key = un.key(p);
+          if (!wait_bounded(m_full, (uint32_t)m_loads & 1u, abort_flag, p.err, kErrBwM)) break;
+          ++m_loads;
+        }
+        if (!wait_bounded(a_full(buf), (uint32_t)(i >> 1) & 1u, abort_flag, p.err, kErrBwA)) break;
+        tc_fence_after();
+        const uint32_t a_tmem = tmem_base + kBwMaxN + (uint32_t)buf * kBwACols;
+        const uint32_t half_bytes = (uint32_t)(p.atoms * kBwAtomBytes), part_bytes = (uint32_t)p.nh * half_bytes;
+        bool ok = true;
+        for (int hf = 0; hf < p.nh; ++hf) {
+          if (!(ok = wait_bounded(d_empty(hf), (uint32_t)(i & 1) ^ 1u, abort_flag, p.err, kErrBwDEmpty))) break;
+          tc_fence_after();
+          const int na = max(1, min(p.hr, d.n_out - (un.t * p.nh + hf) * p.hr));  // a half without rows: its zeros
+          const uint32_t idesc = idesc_bf16(128, (na * d.n_in + 15) / 16 * 16, false, true);
+          const uint32_t d_tmem = tmem_base + (uint32_t)(hf * 128);
+          // operand addresses by one addition each: a descriptor built per MMA took longer than the MMA
+          const uint64_t bd0 = umma_desc(sbase + (uint32_t)hf * half_bytes, kBwAtomBytes, 1024, kSwizzle128B);
+#pragma unroll
+          for (int pr = 0; pr < 6; ++pr) {  // part products, smallest first
+            constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+            const uint64_t bd = bd0 + pb[pr] * (part_bytes >> 4);
+#pragma unroll
+            for (int k = 0; k < kBwK / 16; ++k)
+              if (k < ksteps) mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(pa[pr] * 32 + k * 8), bd + k * 128, idesc, (pr | k) != 0);
+          }
+          mma_commit(d_full(hf));
+        }
+        if (!ok) break;
+        mma_commit(a_empty(buf));
+        un.next(p);
+        if (u + 1 < u1 && un.key(p) != key) mma_commit(m_empty);
+      }
+      mma_commit(drain_bar);
+      wait_drain(drain_bar, 0, p.err, kErrBwDrain);
+    }
+  } else if (warp == kBwLoadWarps + 1) {
+    // ---- copy-out: row (co, a) of the tile is one contiguous run of W ----
+    BwUnit un;
+    un.init(p, u0);
+    const uint32_t run = (uint32_t)rowlen * 2u;
+    int i = 0;
+    bool ok = true;
+    for (int64_t u = u0; u < u1 && ok; ++u, ++i, un.next(p)) {
+      const int co0 = un.pt * p.cpt, nco = min(p.cpt, d.c_out - co0);
+      for (int hf = 0; hf < p.nh && ok; ++hf) {
+        ok = wait_bounded_sleep(stg_full(hf), (uint32_t)i & 1u, abort_flag, p.err, kErrBwStg);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        const int a0 = (un.t * p.nh + hf) * p.hr, na = max(0, min(p.hr, d.n_out - a0));
+        for (int r = lane; r < nco * na; r += 32) {
+          const int col = r / na, al = r - col * na;
+          __nv_bfloat16* dst =
+              p.W + (((int64_t)un.s * d.c_out + co0 + col) * d.n_out + a0 + al) * d.ldW + (int64_t)un.sp * d.in_blk;
+          bulk_store(dst, sbase + stg_off + (uint32_t)hf * p.stg_bytes + (uint32_t)(col * p.hr + al) * run, run);
+        }
+        bulk_commit();
+        bulk_wait_read<0>();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(stg_free(hf));
+      }
+    }
+    // zeros outside the window: a staging buffer cleared once, then copied to every such run
+    const int out_cols = (int)min((int64_t)p.stg_bytes / 2, (int64_t)d.s_in * d.in_blk);  // elements of zeros kept
+    bool any = false;
+    for (int s = 0; s < d.s_out; ++s) any = any || d.win_hi[s] - d.win_lo[s] < d.s_in;
+    if (any && ok) {
+      for (int o = lane * 16; o < out_cols * 2; o += 512) *reinterpret_cast<uint4*>(smem + stg_off + o) = make_uint4(0, 0, 0, 0);
+      fence_proxy_async_smem();
+      __syncwarp();
+      const int per_out = d.c_out * d.n_out;
+      for (int64_t r = (int64_t)blockIdx.x * 32 + lane; r < d.rows_out; r += (int64_t)gridDim.x * 32) {
+        const int s = (int)(r / per_out);
+        for (int side = 0; side < 2; ++side) {
+          const int64_t c0 = side ? (int64_t)max(d.win_hi[s], 0) * d.in_blk : 0;
+          const int64_t c1 = side ? (int64_t)d.s_in * d.in_blk : (int64_t)max(d.win_lo[s], 0) * d.in_blk;
+          for (int64_t c = c0; c < c1; c += out_cols)
+            bulk_store(p.W + r * d.ldW + c, sbase + stg_off, (uint32_t)min((int64_t)out_cols, c1 - c) * 2u);
+        }
+      }
+      bulk_commit();
+    }
+    bulk_wait<0>();
+  } else if (warp < kBwConv0) {
+    // ---- epilogue: lane = channel pair; the two warps of a quarter take alternate rows a ----
+    const int q = warp & 3, h = (warp - kBwEpi0) >> 2, r = q * 32 + lane;
+    const int col = r / d.c_in, ci = r - col * d.c_in;
+    BwUnit un;
+    un.init(p, u0);
+    int i = 0;
+    for (int64_t u = u0; u < u1; ++u, ++i, un.next(p)) {
+      const bool valid = col < p.cpt && un.pt * p.cpt + col < d.c_out;
+      bool ok = true;
+      for (int hf = 0; hf < p.nh; ++hf) {
+        ok = wait_bounded_sleep(stg_free(hf), (uint32_t)(i & 1) ^ 1u, abort_flag, p.err, kErrBwStgFree);
+        ok = ok && wait_bounded_sleep(d_full(hf), (uint32_t)i & 1u, abort_flag, p.err, kErrBwD);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        tc_fence_after();
+        const int na = min(p.hr, d.n_out - (un.t * p.nh + hf) * p.hr);
+        const uint32_t tl = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * 128);
+        for (int al = h; al < na; al += 2) {
+          __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(smem + stg_off + (uint32_t)hf * p.stg_bytes) +
+                               (col * p.hr + al) * rowlen + ci * d.n_in;
+          for (int c = 0; c < d.n_in; c += 48) {
+            uint32_t rv[3][16];
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+              if (c + 16 * j < d.n_in) tmem_ld16_nowait(tl + (uint32_t)(al * d.n_in + c + 16 * j), rv[j]);
+            tmem_wait_ld();
+            if (valid) {
+#pragma unroll
+              for (int j = 0; j < 48; j += 2) {
+                const uint32_t v = pack_bf16x2(rv[j >> 4][j & 15], rv[j >> 4][(j & 15) + 1]);
+                if (c + j < d.n_in) dst[c + j] = __ushort_as_bfloat16((unsigned short)(v & 0xFFFFu));
+                if (c + j + 1 < d.n_in) dst[c + j + 1] = __ushort_as_bfloat16((unsigned short)(v >> 16));
+              }
+            }
+          }
+        }
+        tc_fence_before();
+        fence_proxy_async_smem();  // the staging buffer is read by the copy engine
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(d_empty(hf));
+          mbar_arrive(stg_full(hf));
+        }
+      }
+      if (!ok) break;
+    }
+  } else {
+    // ---- converters: lane = channel pair, kernel points 32 h .. 32 h + 31 ----
+    const int q = warp & 3, h = (warp - kBwConv0) >> 2, r = q * 32 + lane;
+    int slot = 0, i = 0;
+    uint32_t ph = 0;
+    BwUnit un;
+    un.init(p, u0);
+    for (int64_t u = u0; u < u1; ++u, ++i, un.next(p)) {
+      const int buf = i & 1;
+      bool ok = wait_bounded_sleep(w_full(slot), ph, abort_flag, p.err, kErrBwW);
+      ok = ok && wait_bounded_sleep(a_empty(buf), ((uint32_t)(i >> 1) & 1u) ^ 1u, abort_flag, p.err, kErrBwAEmpty);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      const bool valid = r < min(p.cpt, d.c_out - un.pt * p.cpt) * d.c_in;
+      if (32 * h < 16 * ksteps) {
+        const float* src = reinterpret_cast<const float*>(smem + w_off + (uint32_t)slot * p.w_bytes) + r * p.wld + 32 * h;
+        const int kn = valid ? d.K - 32 * h : 0;
+        uint32_t part[3][16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float x = 2 * j < kn ? src[2 * j] : 0.f, y = 2 * j + 1 < kn ? src[2 * j + 1] : 0.f;
+          uint32_t t3[3];
+          split3x2(x, y, t3);
+#pragma unroll
+          for (int t = 0; t < 3; ++t) part[t][j] = t3[t];
+        }
+        const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + kBwMaxN + (uint32_t)buf * kBwACols + 16u * h;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) tmem_st16(at + 32u * t, part[t]);
+        tmem_wait_st();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(w_empty(slot));
+        mbar_arrive(a_full(buf));
+      }
+      if (++slot == p.ring) {
+        slot = 0;
+        ph ^= 1u;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kBwLoadWarps) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
   }
 }
 
@@ -254,37 +444,30 @@ __global__ void __launch_bounds__(kBwThreads, 1)
 // ---------------------------------------------------------------------------
 namespace {
 
-PFN_cuTensorMapEncodeTiled_v12000 bw_encode() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-  });
-  return fn;
-}
+int bw_wld(int K) { return K | 1; }  // odd: the converters' lanes read conflict-free
 
-constexpr size_t kBwSmem = 1024 + kBwOpBytes + 64;
+size_t bw_stg_bytes(int n_in) { return (128 * (size_t)bw_hrows(n_in) * n_in * 2 + 1023) / 1024 * 1024; }
+
+size_t bw_smem(int n_in, int K, int ring) {
+  const size_t img = 3 * (size_t)(bw_halves(n_in) * bw_atoms(n_in)) * kBwAtomBytes;
+  return 1024 + img + bw_halves(n_in) * bw_stg_bytes(n_in) + ring * ((128 * (size_t)bw_wld(K) * 4 + 15) / 16 * 16) +
+         19 * 8 + 64;
+}
 
 }  // namespace
 
 cudaError_t build_w_tables_create(const LscDims& dt, const float* d_M, BuildWTables& t, std::string& err) {
   t = BuildWTables();
-  const int npg = dt.s_out * dt.s_in, nab = dt.n_out * dt.n_in;
-  // the staging tile: up to 128 pairs x bw_max_rows(n_in) rows of n_in entries, in the operand space
-  if (dt.K > kBwK || npg < 1 || nab < 1 || (size_t)kBwTP * bw_max_rows(dt.n_in) * dt.n_in * 2 > kBwOpBytes)
+  if (dt.K > kBwK || dt.n_in < 1 || dt.n_in > kBwMaxN || bw_smem(dt.n_in, dt.K, 1) > kBwSmemLimit)
     return cudaSuccess;  // the CUDA-core build takes these
-  t.npg = npg;
-  t.ldm = (nab + 63) / 64 * 64;
-  const size_t part = (size_t)npg * kBwK * t.ldm;
+  t.npg = dt.m_stride_sp ? dt.s_out * dt.s_in : dt.s_out;
+  const size_t bytes =
+      (size_t)t.npg * bw_tiles(dt.n_in, dt.n_out) * 3 * bw_halves(dt.n_in) * bw_atoms(dt.n_in) * kBwAtomBytes;
   void* mp = nullptr;
-  cudaError_t e = cudaMalloc(&mp, 3 * part * 2);
+  cudaError_t e = cudaMalloc(&mp, bytes);
   if (e == cudaSuccess) {
-    const unsigned blocks = (unsigned)std::min<size_t>((part + 255) / 256, 152 * 8);
-    split_m_kernel<<<blocks, 256>>>(dt, d_M, static_cast<__nv_bfloat16*>(mp), t.ldm, npg);
+    const unsigned blocks = (unsigned)std::min<size_t>((bytes / 6 + 255) / 256, 152 * 8);
+    split_m_kernel<<<blocks, 256>>>(dt, d_M, static_cast<uint8_t*>(mp), t.npg);
     count_launch();
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -306,43 +489,50 @@ void build_w_tables_destroy(BuildWTables& t) {
 }
 
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t) {
-  if (!tc_enabled() || !t.ok || d.K > kBwK || !bw_encode()) return false;
-  if (d.s_out * d.s_in != t.npg || d.c_in < 1 || kBwTP % d.c_in != 0) return false;
+  if (!tc_enabled() || !t.ok || d.c_in < 1 || d.c_in > 128) return false;
+  // rows of a tile leave W in 16-byte granules
+  if (d.in_blk != (int64_t)d.c_in * d.n_in) return false;
   int dev = 0, major = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   return major == 10;
 }
 
-cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, void* W, int* err, cudaStream_t st) {
+cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, const float* b, const float* q, void* W,
+                       float* bias_vec, int* err, cudaStream_t st) {
   TraceScope trace("lsc_build_w_tc", st);
-  const int npg = d.s_out * d.s_in, nab = d.n_out * d.n_in;
-  cudaError_t e;
-  // padding columns between shell blocks stay zero
-  if (d.in_blk != (int64_t)d.c_in * d.n_in) {
-    e = cudaMemsetAsync(W, 0, (size_t)d.rows_out * d.ldW * 2, st);
-    if (e != cudaSuccess) return e;
-  }
-  BwMaps maps;
-  memset(&maps, 0, sizeof maps);
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)t.ldm, (cuuint64_t)(3 * npg * kBwK)};
-    const cuuint64_t strides[1] = {(cuuint64_t)t.ldm * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kBwK};
-    const cuuint32_t es[2] = {1, 1};
-    if (bw_encode()(&maps.b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, t.d_mp, dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
-  // whole runs in 16-byte chunks: W 16-byte aligned, rows and shell blocks of multiples of 8
-  const int rowlen = d.c_in * d.n_in;
-  const int vec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0 && rowlen % 8 == 0 && d.ldW % 8 == 0 && d.in_blk % 8 == 0;
-  e = cudaFuncSetAttribute(build_w_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwSmem);
+  BwParams p;
+  memset(&p, 0, sizeof p);
+  p.d = d;
+  p.w = w;
+  p.img = static_cast<const uint8_t*>(t.d_mp);
+  p.b = b;
+  p.q = q;
+  p.bias = bias_vec;
+  p.W = static_cast<__nv_bfloat16*>(W);
+  p.nh = bw_halves(d.n_in);
+  p.hr = bw_hrows(d.n_in);
+  p.nt = bw_tiles(d.n_in, d.n_out);
+  p.atoms = bw_atoms(d.n_in);
+  p.cpt = 128 / d.c_in;
+  p.nptiles = (d.c_out + p.cpt - 1) / p.cpt;
+  p.wld = bw_wld(d.K);
+  p.pg_per_pair = d.m_stride_sp ? 1 : 0;
+  p.img_bytes = (uint32_t)(3 * p.nh * p.atoms * kBwAtomBytes);
+  p.w_bytes = (uint32_t)((128 * p.wld * 4 + 15) / 16 * 16);
+  p.stg_bytes = (uint32_t)bw_stg_bytes(d.n_in);
+  p.ring = bw_smem(d.n_in, d.K, 2) <= kBwSmemLimit ? 2 : 1;
+  p.err = err;
+  for (int s = 0; s < d.s_out; ++s) p.units += (int64_t)p.nt * std::max(0, d.win_hi[s] - d.win_lo[s]) * p.nptiles;
+  if (p.units == 0) return cudaErrorInvalidValue;
+  // at least 120 KiB so that two CTAs never share an SM (each holds 512 TMEM columns)
+  const size_t smem = std::max<size_t>(120 * 1024, bw_smem(d.n_in, d.K, p.ring));
+  cudaError_t e = cudaFuncSetAttribute(build_w_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int npairs = d.c_out * d.c_in;
-  const dim3 grid((unsigned)((nab + kBwTN - 1) / kBwTN), (unsigned)((npairs + kBwTP - 1) / kBwTP), (unsigned)npg);
-  build_w_tc_kernel<<<grid, kBwThreads, kBwSmem, st>>>(maps, d, w, static_cast<__nv_bfloat16*>(W), vec, err);
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  build_w_tc_kernel<<<(unsigned)std::min<int64_t>(p.units, std::max(1, sms)), kBwThreads, smem, st>>>(p);
   count_launch();
   return cudaGetLastError();
 }

@@ -84,22 +84,21 @@ cudaError_t split_bf16x3(const float* x, int64_t rows, int64_t cols, int64_t ldx
 
 // The LSC forward with SH2Signal in its epilogue (tc_fused.cu): B_s^T of the output basis'
 // shells as the K-major BF16 operator [S][96 directions][64 coefficients], zero-padded.
-// Parts of the collapse matrices M_{s,s'} for the tensor-core operator build: three BF16
-// parts of every shell pair's [64 kernel points (zero past K)][ldm (a,b) entries] block,
-// part q at q * npg * 64 * ldm (ok false: K > 64 or rows too long for the staging tile;
-// the CUDA-core build is used).
+// Parts of the collapse matrices for the tensor-core operator build: per shell (or shell pair)
+// and tile of output rows the three BF16 parts of M as operand images (ok false: more than 64
+// kernel points or tables that do not fit; the CUDA-core build is used).
 struct BuildWTables {
   void* d_mp = nullptr;
-  int npg = 0, ldm = 0;
+  int npg = 0;
   bool ok = false;
 };
 cudaError_t build_w_tables_create(const LscDims& dims_template, const float* d_M, BuildWTables& t, std::string& err);
 void build_w_tables_destroy(BuildWTables& t);
-// The BF16 operator W on the tensor cores (zeros outside the window and in the padding);
-// supported when K <= 64 and c_in divides 128 (the caller takes it only where the
-// forward reads W, i.e. without padding between shell blocks).
+// The BF16 operator W on the tensor cores (zeros outside the window) and, where bias_vec is
+// given, the bias vector; K <= 64, c_in <= 128 and no padding between shell blocks.
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t);
-cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, void* W, int* err, cudaStream_t st);
+cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, const float* b, const float* q, void* W,
+                       float* bias_vec, int* err, cudaStream_t st);
 
 // Parts of the collapse matrices for the weight gradient's reduction on the tensor cores: per
 // shell (or shell pair) and input coefficient b the three BF16 parts of M as operand images (ok

@@ -272,13 +272,14 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
           }
           tc_fence_after();
           const uint32_t a_tmem = tmem_base + kRdDCols + (uint32_t)buf * a_cols;
-          const uint32_t b_src = sbase + (uint32_t)b * p.img_bytes;
+          // operand addresses by one addition each: a descriptor built per MMA took longer than the MMA
+          const uint64_t bd0 = umma_desc(sbase + (uint32_t)b * p.img_bytes, part_bytes, 1024, kSwizzle128B);
           for (int kk = 0; kk < p.ks; ++kk) {
 #pragma unroll
             for (int pr = 0; pr < 6; ++pr) {  // part products, smallest first
               constexpr int pa[6] = {2, 1, 0, 1, 0, 0}, pb[6] = {0, 1, 2, 0, 1, 0};
-              const uint64_t bd = umma_desc(b_src + pb[pr] * part_bytes + kk * 2048, part_bytes, 1024, kSwizzle128B);
-              mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(pa[pr] * 8 * p.ks + kk * 8), bd, idesc, (b | kk | pr) != 0);
+              mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(pa[pr] * 8 * p.ks + kk * 8), bd0 + pb[pr] * (part_bytes >> 4) + kk * 128,
+                          idesc, (b | kk | pr) != 0);
             }
           }
           mma_commit(a_empty(buf));
@@ -442,8 +443,16 @@ __global__ void __launch_bounds__(256) finish_dw_kernel(const __grid_constant__ 
     const bool in = row < p.rows_total && sp >= d.win_lo[s] && sp < d.win_hi[s];
     for (int k = warp; k < d.K; k += 8) {
       float a = 0.f;
-      if (in)
-        for (int z = 0; z < p.nparts; ++z) a += p.dwp[z * p.part_stride + k * p.rows_total + row];
+      if (in) {  // eight parts' loads in flight, summed in order
+        const float* src = p.dwp + k * p.rows_total + row;
+        for (int z0 = 0; z0 < p.nparts; z0 += 8) {
+          float v[8];
+#pragma unroll
+          for (int z = 0; z < 8; ++z) v[z] = z0 + z < p.nparts ? __ldg(src + (z0 + z) * p.part_stride) : 0.f;
+#pragma unroll
+          for (int z = 0; z < 8; ++z) a += v[z];
+        }
+      }
       t[k][lane] = a;
     }
     __syncthreads();
