@@ -160,7 +160,13 @@ def lsc_backward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, d_out: t
     x = as_act(x)
     d_out = as_act(d_out.to(x.dtype))
     n_vox = x.shape[1]
-    d_in = empty_act(x.shape[0], n_vox, x.dtype, x.device) if need_input else None
+    d_in = None
+    if need_input:  # the call takes one row stride for both
+        if x.stride(0) > 2 * padded_ld(n_vox):
+            x = empty_act(x.shape[0], n_vox, x.dtype, x.device).copy_(x)
+        d_in = torch.empty((x.shape[0], x.stride(0)), dtype=x.dtype, device=x.device)
+        if x.stride(0) != n_vox:
+            d_in = d_in[:, :n_vox]
     w = w.detach().contiguous().float()
     dw = torch.empty_like(w) if need_weight else None
     db = torch.empty((c_out, geom.s_out), dtype=torch.float32, device=x.device) if need_bias else None
