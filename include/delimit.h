@@ -171,6 +171,16 @@ delimit_status delimit_sh2signal_backward(const delimit_sh_basis* basis, const v
                                           int64_t n_vox, int channels, int64_t ld_sig, int64_t ld_sh,
                                           delimit_dtype in_t, delimit_dtype out_t, void* stream);
 
+/* One of the four transforms (kind 0: delimit_signal2sh, 1: delimit_sh2signal, 2:
+ * delimit_signal2sh_backward, 3: delimit_sh2signal_backward) of an F32 input whose pointer and
+ * row stride need only its elements' alignment (a volume with any number of voxels as it
+ * lies).  The output follows the 16-byte rule.  UNSUPPORTED where the input breaks the 16-byte
+ * rule and no tensor-core FP32 kernel takes the call (the caller copies it into padded rows
+ * then); otherwise as those calls. */
+delimit_status delimit_transform_unaligned(const delimit_sh_basis* basis, int kind, const void* x, void* y,
+                                           int64_t n_vox, int channels, int64_t ld_x, int64_t ld_y,
+                                           delimit_dtype in_t, delimit_dtype out_t, void* stream);
+
 /* ------------------------------------------------------------------------ */
 /* Local spherical convolution (Sec. 2.3; multi-shell form of Sec. 2.3.1).   */
 /* ------------------------------------------------------------------------ */

@@ -59,6 +59,8 @@ SIGNATURES = {
     "delimit_sh2signal": (C.c_int, [_vp, _vp, _vp, _i64, C.c_int, _i64, _i64, C.c_int, C.c_int, _vp]),
     "delimit_signal2sh_backward": (C.c_int, [_vp, _vp, _vp, _i64, C.c_int, _i64, _i64, C.c_int, C.c_int, _vp]),
     "delimit_sh2signal_backward": (C.c_int, [_vp, _vp, _vp, _i64, C.c_int, _i64, _i64, C.c_int, C.c_int, _vp]),
+    "delimit_transform_unaligned": (C.c_int, [_vp, C.c_int, _vp, _vp, _i64, C.c_int, _i64, _i64, C.c_int, C.c_int,
+                                              _vp]),
     "delimit_lsc_geometry_create": (C.c_int, [_vp, C.c_int, C.c_int, C.c_double, C.c_int, C.c_int, C.c_int,
                                               C.c_uint, C.POINTER(_vp)]),
     "delimit_lsc_geometry_destroy": (C.c_int, [_vp]),

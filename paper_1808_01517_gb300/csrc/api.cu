@@ -299,7 +299,7 @@ static delimit_status check_act(const void* p, int64_t ld, int64_t n_vox, delimi
 
 static delimit_status run_transform(const delimit_sh_basis* b, const void* X, void* Y, int64_t n_vox, int C,
                                     int64_t ldx, int64_t ldy, delimit_dtype in_t, delimit_dtype out_t, void* stream,
-                                    TransformKind kind) {
+                                    TransformKind kind, bool any_input = false) {
   if (!b) return fail(DELIMIT_ERR_INVALID_ARG, "basis is NULL");
   if (!b->on_device) return fail(DELIMIT_ERR_INVALID_ARG, "basis was created with DELIMIT_HOST_ONLY");
   if (!b->h.has_pinv && (kind == kS2SH || kind == kS2SH_BWD))
@@ -309,7 +309,16 @@ static delimit_status run_transform(const delimit_sh_basis* b, const void* X, vo
   if (n_vox == 0) return DELIMIT_OK;
   delimit_status st = check_device(b->device);
   if (st != DELIMIT_OK) return st;
-  if ((st = check_act(X, ldx, n_vox, in_t, "input")) != DELIMIT_OK) return st;
+  const bool aligned = !any_input || (aligned16(X) && (ldx * elem_size(in_t)) % 16 == 0);
+  if (aligned) {
+    if ((st = check_act(X, ldx, n_vox, in_t, "input")) != DELIMIT_OK) return st;
+  } else {
+    if (!X) return fail(DELIMIT_ERR_INVALID_ARG, "input is NULL");
+    if (ldx < n_vox) return fail(DELIMIT_ERR_INVALID_ARG, "input: ld < n_vox");
+    if (reinterpret_cast<uintptr_t>(X) % elem_size(in_t)) return fail(DELIMIT_ERR_ALIGNMENT, "input: pointer off its elements");
+    if (in_t != DELIMIT_F32 || !tc_transform_f32_supported(b->tc, kind, out_t))
+      return fail(DELIMIT_ERR_UNSUPPORTED, "unaligned input: F32 on the tensor-core kernels only");
+  }
   if ((st = check_act(Y, ldy, n_vox, out_t, "output")) != DELIMIT_OK) return st;
   const int N = b->h.N, S = int(b->h.shells.size());
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
@@ -322,7 +331,7 @@ static delimit_status run_transform(const delimit_sh_basis* b, const void* X, vo
   // FP32 input: three-part BF16 splits made in shared memory, six part products
   if (in_t == DELIMIT_F32 && tc_transform_f32_supported(b->tc, kind, out_t)) {
     cudaError_t e = tc_transform_f32_launch(b->tc, kind, static_cast<const float*>(X), Y, n_vox, C, ldx, ldy, out_t,
-                                            b->err_word, cs);
+                                            aligned, b->err_word, cs);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core FP32 transform launch");
     return DELIMIT_OK;
   }
@@ -362,6 +371,13 @@ extern "C" {
 delimit_status delimit_signal2sh(const delimit_sh_basis* b, const void* sig, void* sh, int64_t n_vox, int channels,
                                  int64_t ld_sig, int64_t ld_sh, delimit_dtype in_t, delimit_dtype out_t, void* stream) {
   return run_transform(b, sig, sh, n_vox, channels, ld_sig, ld_sh, in_t, out_t, stream, kS2SH);
+}
+
+delimit_status delimit_transform_unaligned(const delimit_sh_basis* b, int kind, const void* x, void* y, int64_t n_vox,
+                                           int channels, int64_t ld_x, int64_t ld_y, delimit_dtype in_t,
+                                           delimit_dtype out_t, void* stream) {
+  if (kind < kS2SH || kind > kSH2S_BWD) return fail(DELIMIT_ERR_INVALID_ARG, "unknown transform");
+  return run_transform(b, x, y, n_vox, channels, ld_x, ld_y, in_t, out_t, stream, TransformKind(kind), true);
 }
 
 delimit_status delimit_signal2sh_gather(const delimit_sh_basis* b, const void* dwi, int64_t ld_dwi, int64_t n_src,

@@ -20,10 +20,10 @@ struct TcBasisTables {
   bool ok = false;
   // FP32 activations: three BF16 parts of every operator (T = T0 + T1 + T2) side by side
   // along the output axis, [kpad][npad3] per shell and kind at byte offset off3 in d_mem3,
-  // part q from column q * npad3 / 3 (whole 64-column atoms)
+  // part q from column q * pstride3
   void* d_mem3 = nullptr;
   size_t off3[kMaxGroups][4] = {};
-  int npad3[kMaxGroups][4] = {};
+  int npad3[kMaxGroups][4] = {}, pstride3[kMaxGroups][4] = {};
   bool ok3 = false;
 };
 
@@ -37,10 +37,12 @@ bool tc_transform_supported(const TcBasisTables& t, int kind, int64_t ldx, int64
 cudaError_t tc_transform_launch(const TcBasisTables& t, int kind, const void* X, void* Y, int64_t n_vox, int C,
                                 int64_t ldx, int64_t ldy, int out_t, int* err_word, cudaStream_t st);
 // FP32 input (out_t: 0 = F32, 1 = BF16): each value split into three BF16 parts in shared
-// memory, six part products accumulated in FP32 on the tensor cores
+// memory, six part products accumulated in FP32 on the tensor cores; aligned: X and its rows
+// start on 16-byte boundaries (else plain copies in place of TMA)
 bool tc_transform_f32_supported(const TcBasisTables& t, int kind, int out_t);
 cudaError_t tc_transform_f32_launch(const TcBasisTables& t, int kind, const float* X, void* Y, int64_t n_vox, int C,
-                                    int64_t ldx, int64_t ldy, int out_t, int* err_word, cudaStream_t st);
+                                    int64_t ldx, int64_t ldy, int out_t, bool aligned, int* err_word,
+                                    cudaStream_t st);
 
 // LSC GEMMs (BF16 activations, FP32 accumulation in TMEM).
 // FP32 activations: every operand is passed as three BF16 parts (split_bf16x3), part p

@@ -39,13 +39,17 @@ def empty_act(rows: int, n_vox: int, dtype, device="cuda") -> torch.Tensor:
     return torch.empty((rows, padded_ld(n_vox)), dtype=dtype, device=device)[:, :n_vox]
 
 
+def _is_act(x: torch.Tensor) -> bool:
+    """Unit voxel stride, rows that do not overlap and start on 16-byte boundaries."""
+    return x.stride(1) == 1 and (x.stride(0) * x.element_size()) % 16 == 0 and x.data_ptr() % 16 == 0 \
+        and x.stride(0) >= x.shape[1]
+
+
 def as_act(x: torch.Tensor) -> torch.Tensor:
     """x as a 2-D activation with unit voxel stride and an aligned row stride (copies if needed)."""
     if x.dim() != 2:
         raise ValueError("activations are 2-D [features, voxels]")
-    ok = x.stride(1) == 1 and (x.stride(0) * x.element_size()) % 16 == 0 and x.data_ptr() % 16 == 0 \
-        and x.stride(0) >= x.shape[1]
-    if ok:
+    if _is_act(x):
         return x
     y = empty_act(x.shape[0], x.shape[1], x.dtype, x.device)
     y.copy_(x)
@@ -61,12 +65,17 @@ _TRANSFORMS = {
     "signal2sh_backward": "delimit_signal2sh_backward",
     "sh2signal_backward": "delimit_sh2signal_backward",
 }
+_KINDS = {k: i for i, k in enumerate(_TRANSFORMS)}
 
 
 def transform(kind: str, basis: L.SHBasis, x: torch.Tensor, channels: int, out_dtype=None,
               out: torch.Tensor | None = None) -> torch.Tensor:
     """One of the four transforms; output rows follow the library's row order."""
-    x = as_act(x)
+    # rows of FP32 voxels off the 16-byte boundaries are read as they lie where a kernel takes them
+    as_lies = x.dim() == 2 and x.dtype is torch.float32 and x.is_cuda and x.stride(1) == 1 \
+        and x.stride(0) >= x.shape[1] and not _is_act(x)
+    if not as_lies:
+        x = as_act(x)
     n_vox = x.shape[1]
     to_sh = kind in ("signal2sh", "sh2signal_backward")
     rows_out = basis.n_shells * channels * basis.n_coef if to_sh else channels * basis.n_dirs
@@ -76,6 +85,13 @@ def transform(kind: str, basis: L.SHBasis, x: torch.Tensor, channels: int, out_d
     od = out_dtype or x.dtype
     if out is None:
         out = empty_act(rows_out, n_vox, od, x.device)
+    if as_lies:
+        st = L.get().delimit_transform_unaligned(basis.handle, _KINDS[kind], x.data_ptr(), out.data_ptr(), n_vox,
+                                                 channels, x.stride(0), out.stride(0), _code(x), _code(out), _stream())
+        if st != L.ERR_UNSUPPORTED:
+            L.check(st, "delimit_transform_unaligned")
+            return out
+        x = as_act(x)
     fn = getattr(L.get(), _TRANSFORMS[kind])
     L.check(fn(basis.handle, x.data_ptr(), out.data_ptr(), n_vox, channels, x.stride(0), out.stride(0), _code(x),
                _code(out), _stream()), _TRANSFORMS[kind])
