@@ -102,6 +102,7 @@ __host__ __device__ inline int k_chunks(int nkb, int chunk_kb) { return nkb > 0 
 struct VoxParams {
   VoxGroup g[kMaxGroups];
   int n_groups, m_tiles, tiles_per_m;
+  int m_units, m_group;  // voxel tiles (tile pairs for clusters of two), and how many are walked together
   int b_kmajor;  // operator stored [N rows][K contiguous] (K-major) instead of [K rows][N contiguous]
   int n_terms;   // 1 (BF16 operands) or kSplitTerms (three-part BF16 splits of FP32 operands)
   int chunk_kb;  // K blocks per accumulation chunk (> 0; chunks after the first are added in the epilogue)
@@ -112,9 +113,24 @@ struct VoxParams {
   int* err;
 };
 
+// Tile order: kVoxGroup voxel tiles are walked together, operator tile by operator tile (voxel tile
+// fastest), then the next group; persistent clusters take tiles round-robin.  The 76 tiles in flight
+// then cover about 16 voxel x 5 operator tiles and read half the operand bytes from L2 and DRAM
+// that 2 x 36 tiles do (64 -> 64 channels: an operator of 116 MB per 76 tiles), and the tiles of
+// one operator tile, equal in K, fill the rounds evenly.  64 -> 64 channels, 8,192 voxels: forward
+// 0.645 -> 0.589 ms, input gradient 0.654 -> 0.599 (groups of 4: 0.601 / 0.610, 32: 0.610 / 0.619);
+// 16 -> 64 channels, 65,536 voxels, where the operator fits L2: 1.240 -> 1.232 and 1.164 -> 1.168.
+constexpr int kVoxGroup = 16;
+// up to this K a tile's time is its output's stores, not its operands: voxel tiles one by one
+constexpr int kShortK = 1024;
 __device__ __forceinline__ void vox_decode(const VoxParams& p, int64_t t, int& g, int& mt, int& nt) {
-  mt = (int)(t / p.tiles_per_m);
-  int r = (int)(t % p.tiles_per_m);
+  const int64_t per = (int64_t)p.m_group * p.tiles_per_m;
+  const int m0 = (int)(t / per) * p.m_group, gm = min(p.m_group, p.m_units - m0);
+  int r = (int)(t % per);
+  mt = r / gm;
+  const int m = m0 + r - mt * gm;
+  r = mt;
+  mt = m;
   g = 0;
   while (r >= p.g[g].n_tiles) {
     r -= p.g[g].n_tiles;
@@ -288,11 +304,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
+    const bool bk = p.b_kmajor != 0;
+    // Operand descriptors of stage 0; a stage, and a k-step within it, lies a constant further on (16-byte
+    // units, no carry out of the address field: shared memory ends below 2^18).  One addition per
+    // operand: a descriptor built per MMA kept this thread near the MMA rate (forward 1.23 -> 1.18 ms at
+    // 16 -> 64 channels, 65,536 voxels, 0.566 -> 0.548 at 64 -> 64, 8,192).
+    // MN-major, 128-byte swizzle: 64-element MN atoms kBoxBytes apart (LBO), 8-row K groups 1024 B
+    // apart (SBO); 16 K rows = 2048 B per MMA.  K-major operator: rows 128 B apart, 8-row groups
+    // 1024 B apart, 16 K = 32 B per MMA.
+    const uint64_t ad0 = umma_desc(sbase, kBoxBytes, 1024, kSwizzle128B);
+    const uint64_t bd0 = bk ? umma_desc(sbase + A_BYTES, 16, 1024, kSwizzle128B)
+                            : umma_desc(sbase + A_BYTES, kBoxBytes, 1024, kSwizzle128B);
+    const uint32_t bstep = bk ? 32 / 16 : 2048 / 16;
     for (int64_t t = t_first; ok && t < p.total_tiles && !*abort_flag; t += t_step) {
       int g, mt, nt;
       vox_decode(p, t, g, mt, nt);
       const int nkb = (p.g[g].K + kBK - 1) / kBK;
-      const bool bk = p.b_kmajor != 0;
       const uint32_t idesc = idesc_bf16(128 * CL, nt == p.g[g].n_tiles - 1 ? p.g[g].bn_last : BN, true, !bk);
       const int nch = SPLIT ? k_chunks(nkb, chunk_kb) : 1;
       for (int c = 0; c < nch; ++c) {
@@ -310,19 +337,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           tc_fence_after();
-          const uint32_t a_src = sbase + stage * STAGE_BYTES, b_src = a_src + A_BYTES;
+          const uint32_t soff = (uint32_t)stage * (STAGE_BYTES / 16);
+          const uint64_t ad = ad0 + soff, bd = bd0 + soff;
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k) {
-            // MN-major, 128-byte swizzle: 64-element MN atoms kBoxBytes apart (LBO),
-            // 8-row K groups 1024 B apart (SBO); 16 K rows = 2048 B per MMA.  K-major
-            // operator: rows 128 B apart, 8-row groups 1024 B apart, 16 K = 32 B per MMA.
-            const uint64_t ad = umma_desc(a_src + k * 2048, kBoxBytes, 1024, kSwizzle128B);
-            const uint64_t bd = bk ? umma_desc(b_src + k * 32, 16, 1024, kSwizzle128B)
-                                   : umma_desc(b_src + k * 2048, kBoxBytes, 1024, kSwizzle128B);
             if (CL > 1)
-              mma_bf16_pair(d_tmem, ad, bd, idesc, (kb | k) != 0);
+              mma_bf16_pair(d_tmem, ad + k * (2048 / 16), bd + k * bstep, idesc, (kb | k) != 0);
             else
-              mma_bf16(d_tmem, ad, bd, idesc, (kb | k) != 0);
+              mma_bf16(d_tmem, ad + k * (2048 / 16), bd + k * bstep, idesc, (kb | k) != 0);
           }
           if (CL > 1)
             mma_commit_pair_mc(empty_bar(stage), 0x3);  // both CTAs' producers refill this stage
@@ -584,6 +606,7 @@ struct WgParams {
   int n_groups, splits;
   int n_terms;   // 1 (BF16 operands) or kSplitTerms (three-part splits of FP32 operands)
   int chunk_kb;  // voxel blocks of 64 per accumulation chunk (> 0)
+  int m_group;   // row tiles walked together, column tile by column tile
   int64_t tiles_per_split, total_tiles, vps, n_vox, ldp, split_stride;
   int64_t ones_col;  // column of the row sums (rows_in)
   // element (row r, column c) of a split's partial at r * p_rs + c * p_cs: (ldp, 1), or (1, ldp)
@@ -594,6 +617,12 @@ struct WgParams {
   int* err;
 };
 
+// Row tiles of a weight gradient whose column tiles outnumber this are walked kVoxGroup at a time,
+// column tile by column tile: the tiles in flight cover about 12 x 6 in place of 2 x 36 (64 -> 64
+// channels, 24 to 36 column tiles: 0.604 -> 0.585 ms); with fewer column tiles they are near
+// square as they come (16 -> 64 channels, 6 to 9: 1.104 ms against 1.113 walked together).
+constexpr int kWgradRowOfTiles = 12;
+
 __device__ __forceinline__ void wg_decode(const WgParams& p, int64_t t, int& split, int& g, int& mt, int& nt) {
   split = (int)(t / p.tiles_per_split);
   int64_t r = t % p.tiles_per_split;
@@ -602,8 +631,10 @@ __device__ __forceinline__ void wg_decode(const WgParams& p, int64_t t, int& spl
     r -= (int64_t)p.g[g].m_tiles * p.g[g].n_tiles;
     ++g;
   }
-  mt = (int)(r / p.g[g].n_tiles);
-  nt = (int)(r % p.g[g].n_tiles);
+  const int per = p.m_group * p.g[g].n_tiles, m0 = (int)(r / per) * p.m_group;
+  const int gm = min(p.m_group, p.g[g].m_tiles - m0), rr = (int)(r % per);
+  nt = rr / gm;
+  mt = m0 + rr - nt * gm;
 }
 
 template <int BN, int CL, bool SPLIT>
@@ -762,6 +793,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
+    // K-major, 128-byte swizzle: rows 128 B apart, 8-row groups 1024 B apart (SBO); 16 voxels = 32 B
+    // per MMA inside the swizzle atom.  One addition per stage and k-step, as in the GEMM above.
+    const uint64_t ad0 = umma_desc(sbase, 16, 1024, kSwizzle128B), bd0 = umma_desc(sbase + A_BYTES, 16, 1024, kSwizzle128B);
     for (int64_t t = t_first; ok && t < p.total_tiles && !*abort_flag; t += t_step) {
       int split, g, mt, nt;
       wg_decode(p, t, split, g, mt, nt);
@@ -784,17 +818,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           tc_fence_after();
-          const uint32_t a_src = sbase + stage * STAGE_BYTES, b_src = a_src + A_BYTES;
+          const uint32_t soff = (uint32_t)stage * (STAGE_BYTES / 16);
+          const uint64_t ad = ad0 + soff, bd = bd0 + soff;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            // K-major, 128-byte swizzle: rows 128 B apart, 8-row groups 1024 B apart (SBO);
-            // 16 voxels = 32 B per MMA inside the swizzle atom.
-            const uint64_t ad = umma_desc(a_src + k * 32, 16, 1024, kSwizzle128B);
-            const uint64_t bd = umma_desc(b_src + k * 32, 16, 1024, kSwizzle128B);
             if (CL > 1)
-              mma_bf16_pair(d_tmem, ad, bd, idesc, (kb | k) != 0);
+              mma_bf16_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0);
             else
-              mma_bf16(d_tmem, ad, bd, idesc, (kb | k) != 0);
+              mma_bf16(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0);
           }
           if (CL > 1)
             mma_commit_pair_mc(empty_bar(stage), 0x3);
@@ -1216,10 +1247,12 @@ cudaError_t launch_vox_cl(const CUtensorMap& ma, const CUtensorMap& mb, const CU
   if constexpr ((BN / 2) % 8 == 0) {
     // a pair splits the operator columns: whole 64-column atoms for an MN-major operator
     if (cl > 1 && (p.b_kmajor || (BN / 2) % 64 == 0)) {
-      p.total_tiles = (int64_t)((p.m_tiles + 1) / 2) * p.tiles_per_m;
+      p.m_units = (p.m_tiles + 1) / 2;
+      p.total_tiles = (int64_t)p.m_units * p.tiles_per_m;
       return launch_vox<BN, STAGED, 2, SPLIT>(ma, mb, my, p, st);
     }
   }
+  p.m_units = p.m_tiles;
   p.total_tiles = (int64_t)p.m_tiles * p.tiles_per_m;
   return launch_vox<BN, STAGED, 1, SPLIT>(ma, mb, my, p, st);
 }
@@ -1261,11 +1294,17 @@ cudaError_t run_vox(const CUtensorMap& ma, const OperatorView& B, VoxParams& p, 
     return cudaErrorInvalidValue;
   if (p.n_terms < 1) p.n_terms = 1;
   if (p.chunk_kb < 1) p.chunk_kb = 1 << 24;
+  int k_max = 0;
+  for (int i = 0; i < p.n_groups; ++i) k_max = std::max(k_max, p.g[i].K);
+  p.m_group = k_max > kShortK ? kVoxGroup : 1;
   if (p.Yf) staged_ok = false;  // FP32 outputs leave through direct stores
   p.b_kmajor = B.kmajor ? 1 : 0;
   p.tiles_per_m = 0;
   bool same_n = true;
-  const int atom = 64 * (cl > 1 && (bn / 2) % 64 == 0 ? 2 : 1);  // last-tile granularity
+  // last-tile granularity: whole 64-column atoms per CTA of an MN-major operator; a K-major one only
+  // needs whole 8-row groups per CTA and N in steps of 16 per CTA (2,880 = 11 x 256 + 64 columns: the
+  // last tile 64 wide in place of 128, 2 % of the products)
+  const int atom = B.kmajor ? 16 * cl : 64 * (cl > 1 && (bn / 2) % 64 == 0 ? 2 : 1);
   for (int i = 0; i < p.n_groups; ++i) {
     p.g[i].n_tiles = (p.g[i].N + bn - 1) / bn;
     const int rem = p.g[i].N - (p.g[i].n_tiles - 1) * bn;
@@ -1405,8 +1444,12 @@ cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const 
   p.bias = nullptr;
   p.err = err;
   const int bn = kmajor ? kDgradBN : pick_bn(Ns, d.s_in);
-  return run_vox(ma, B, p, bn, false,
-                 gemm_cluster(2), dX, lddx, st);
+  // A short K leaves a tile's time to its stores: whole row segments through the staging tile (64 -> 1
+  // channels at 8,192 voxels, K = 90 .. 135: 0.059 ms against 0.186 with a lane per voxel); a long one
+  // hides them under the next tile's MMAs and takes the deeper ring instead.
+  int k_max = 0;
+  for (int sp = 0; sp < d.s_in; ++sp) k_max = std::max(k_max, p.g[sp].K);
+  return run_vox(ma, B, p, bn, bn % 64 == 0 && k_max <= kShortK, gemm_cluster(2), dX, lddx, st);
 }
 
 template <int BN, int S, int CL, bool SPLIT>
@@ -1449,6 +1492,9 @@ cudaError_t tc_lsc_wgrad(const LscDims& d, const void* dY, const void* X, float*
   p.n_groups = d.s_out;
   p.n_terms = parts.on() ? kSplitTerms : 1;
   p.chunk_kb = parts.on() ? kSplitChunkKb : (1 << 24);
+  int n_tiles = 0;
+  for (int s = 0; s < d.s_out; ++s) n_tiles = std::max(n_tiles, p.g[s].n_tiles);
+  p.m_group = n_tiles > kWgradRowOfTiles ? kVoxGroup : 1;
   p.splits = splits;
   p.total_tiles = p.tiles_per_split * splits;
   p.vps = vps;
