@@ -108,7 +108,7 @@ struct BwParams {
   int64_t units;
   int nh, hr, nt, atoms, cpt, nptiles, ring, wld;  // cpt: output channels per tile; wld: odd row length of w in the ring
   int pg_per_pair;
-  uint32_t img_bytes, w_bytes, stg_bytes;  // stg_bytes: one half's staging buffer
+  uint32_t img_bytes, w_bytes, stg_bytes;  // stg_bytes: one half's staging buffer, rows of in_blk elements
   int* err;
 };
 
@@ -197,13 +197,18 @@ __global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_
       p.bias[r] = p.b ? p.b[co * d.s_out + s] * p.q[s * d.n_out + aa] : 0.f;
     }
   }
+  const int rowlen = (int)d.in_blk;  // a row run of W with its padding, which the staging buffers keep at zero
+  if (rowlen != d.c_in * d.n_in) {
+    for (uint32_t o = threadIdx.x * 16; o < p.nh * p.stg_bytes; o += kBwThreads * 16)
+      *reinterpret_cast<uint4*>(smem + stg_off + o) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int64_t u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
   const int ksteps = (d.K + 15) / 16;
-  const int rowlen = d.c_in * d.n_in;
 
   if (warp < kBwLoadWarps) {
     // ---- loaders: 32 of the tile's 128 pairs each; the first loads the M image too ----
@@ -309,11 +314,14 @@ __global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_
         ok = wait_bounded_sleep(stg_full(hf), (uint32_t)i & 1u, abort_flag, p.err, kErrBwStg);
         if (!(ok = __all_sync(0xffffffffu, ok))) break;
         const int a0 = (un.t * p.nh + hf) * p.hr, na = max(0, min(p.hr, d.n_out - a0));
-        for (int r = lane; r < nco * na; r += 32) {
-          const int col = r / na, al = r - col * na;
+        // consecutive rows a are contiguous in W too when it holds one shell block: one copy per channel
+        const int rows = d.ldW == rowlen ? na : 1, runs = na / max(rows, 1);
+        for (int r = lane; r < nco * runs; r += 32) {
+          const int col = r / runs, al = r - col * runs;
           __nv_bfloat16* dst =
               p.W + (((int64_t)un.s * d.c_out + co0 + col) * d.n_out + a0 + al) * d.ldW + (int64_t)un.sp * d.in_blk;
-          bulk_store(dst, sbase + stg_off + (uint32_t)hf * p.stg_bytes + (uint32_t)(col * p.hr + al) * run, run);
+          bulk_store(dst, sbase + stg_off + (uint32_t)hf * p.stg_bytes + (uint32_t)(col * p.hr + al) * run,
+                     (uint32_t)rows * run);
         }
         bulk_commit();
         bulk_wait_read<0>();
@@ -446,11 +454,14 @@ namespace {
 
 int bw_wld(int K) { return K | 1; }  // odd: the converters' lanes read conflict-free
 
-size_t bw_stg_bytes(int n_in) { return (128 * (size_t)bw_hrows(n_in) * n_in * 2 + 1023) / 1024 * 1024; }
+// a half's staging buffer: 128 / c_in channels x its rows, in_blk elements each
+size_t bw_stg_bytes(int n_in, int c_in, int64_t in_blk) {
+  return ((size_t)(128 / c_in) * bw_hrows(n_in) * in_blk * 2 + 1023) / 1024 * 1024;
+}
 
-size_t bw_smem(int n_in, int K, int ring) {
+size_t bw_smem(int n_in, int c_in, int64_t in_blk, int K, int ring) {
   const size_t img = 3 * (size_t)(bw_halves(n_in) * bw_atoms(n_in)) * kBwAtomBytes;
-  return 1024 + img + bw_halves(n_in) * bw_stg_bytes(n_in) + ring * ((128 * (size_t)bw_wld(K) * 4 + 15) / 16 * 16) +
+  return 1024 + img + bw_halves(n_in) * bw_stg_bytes(n_in, c_in, in_blk) + ring * ((128 * (size_t)bw_wld(K) * 4 + 15) / 16 * 16) +
          19 * 8 + 64;
 }
 
@@ -458,8 +469,7 @@ size_t bw_smem(int n_in, int K, int ring) {
 
 cudaError_t build_w_tables_create(const LscDims& dt, const float* d_M, BuildWTables& t, std::string& err) {
   t = BuildWTables();
-  if (dt.K > kBwK || dt.n_in < 1 || dt.n_in > kBwMaxN || bw_smem(dt.n_in, dt.K, 1) > kBwSmemLimit)
-    return cudaSuccess;  // the CUDA-core build takes these
+  if (dt.K > kBwK || dt.n_in < 1 || dt.n_in > kBwMaxN) return cudaSuccess;  // the CUDA-core build takes these
   t.npg = dt.m_stride_sp ? dt.s_out * dt.s_in : dt.s_out;
   const size_t bytes =
       (size_t)t.npg * bw_tiles(dt.n_in, dt.n_out) * 3 * bw_halves(dt.n_in) * bw_atoms(dt.n_in) * kBwAtomBytes;
@@ -490,8 +500,7 @@ void build_w_tables_destroy(BuildWTables& t) {
 
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t) {
   if (!tc_enabled() || !t.ok || d.c_in < 1 || d.c_in > 128) return false;
-  // rows of a tile leave W in 16-byte granules
-  if (d.in_blk != (int64_t)d.c_in * d.n_in) return false;
+  if (bw_smem(d.n_in, d.c_in, d.in_blk, d.K, 1) > kBwSmemLimit) return false;
   int dev = 0, major = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
@@ -520,13 +529,13 @@ cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, 
   p.pg_per_pair = d.m_stride_sp ? 1 : 0;
   p.img_bytes = (uint32_t)(3 * p.nh * p.atoms * kBwAtomBytes);
   p.w_bytes = (uint32_t)((128 * p.wld * 4 + 15) / 16 * 16);
-  p.stg_bytes = (uint32_t)bw_stg_bytes(d.n_in);
-  p.ring = bw_smem(d.n_in, d.K, 2) <= kBwSmemLimit ? 2 : 1;
+  p.stg_bytes = (uint32_t)bw_stg_bytes(d.n_in, d.c_in, d.in_blk);
+  p.ring = bw_smem(d.n_in, d.c_in, d.in_blk, d.K, 2) <= kBwSmemLimit ? 2 : 1;
   p.err = err;
   for (int s = 0; s < d.s_out; ++s) p.units += (int64_t)p.nt * std::max(0, d.win_hi[s] - d.win_lo[s]) * p.nptiles;
   if (p.units == 0) return cudaErrorInvalidValue;
   // at least 120 KiB so that two CTAs never share an SM (each holds 512 TMEM columns)
-  const size_t smem = std::max<size_t>(120 * 1024, bw_smem(d.n_in, d.K, p.ring));
+  const size_t smem = std::max<size_t>(120 * 1024, bw_smem(d.n_in, d.c_in, d.in_blk, d.K, p.ring));
   cudaError_t e = cudaFuncSetAttribute(build_w_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 1;

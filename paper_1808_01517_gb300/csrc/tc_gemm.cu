@@ -1354,7 +1354,9 @@ bool tc_gemm_supported(const LscDims& d, int64_t n_vox, int64_t ld_in, int64_t l
   return true;
 }
 
-bool tc_forward_reads_w(const LscDims& d) { return d.in_blk == (int64_t)d.c_in * d.n_in; }
+// Without padding between shell blocks, or with one block only (its padding lies past the last
+// input row: zeros in W against rows that read as zero), W's columns are X's rows.
+bool tc_forward_reads_w(const LscDims& d) { return d.in_blk == (int64_t)d.c_in * d.n_in || d.s_in == 1; }
 
 bool tc_dgrad_reads_wt(const LscDims& d) {
   return d.out_blk == (int64_t)d.c_out * d.n_out && ((int64_t)d.c_in * d.n_in) % kDgradBN == 0;
