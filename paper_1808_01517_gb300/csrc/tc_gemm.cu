@@ -968,12 +968,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ---------------------------------------------------------------------------
 // host side
-// Row sums of dY per voxel split (the bias-gradient column of the weight gradient).
-__device__ __forceinline__ float to_f32(float v) { return v; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-template <typename T>
-__global__ void __launch_bounds__(256) rowsum_kernel(const T* __restrict__ dY, int64_t lddy, int64_t rows,
+// Row sums of a BF16 dY per voxel split (the bias-gradient column of the weight gradient).
+__global__ void __launch_bounds__(256) rowsum_kernel(const __nv_bfloat16* __restrict__ dY, int64_t lddy, int64_t rows,
                                                      int64_t n_vox, int64_t vps, int splits, float* __restrict__ P,
                                                      int64_t rs, int64_t split_stride, int64_t col_off) {
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
@@ -982,25 +978,20 @@ __global__ void __launch_bounds__(256) rowsum_kernel(const T* __restrict__ dY, i
   const int64_t row = wid / splits;
   const int split = (int)(wid % splits);
   const int64_t vs = (int64_t)split * vps, ve = min(n_vox, vs + vps);
-  const T* r = dY + row * lddy;
+  const __nv_bfloat16* r = dY + row * lddy;
   float acc = 0.f;
   // vs is a multiple of 128 and rows are 16-byte aligned: 16-byte vectors up to the last full one
-  constexpr int VE = 16 / sizeof(T);
-  const int64_t vend = vs + ((ve - vs) / VE) * VE;
-  for (int64_t v = vs + (int64_t)lane * VE; v < vend; v += 32 * VE) {
+  const int64_t vend = vs + (ve - vs) / 8 * 8;
+  for (int64_t v = vs + (int64_t)lane * 8; v < vend; v += 32 * 8) {
     const uint4 u = *reinterpret_cast<const uint4*>(r + v);
-    if constexpr (sizeof(T) == 2) {
-      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 f = __bfloat1622float2(h[i]);
-        acc += f.x + f.y;
-      }
-    } else {
-      acc += (__uint_as_float(u.x) + __uint_as_float(u.y)) + (__uint_as_float(u.z) + __uint_as_float(u.w));
+    for (int i = 0; i < 4; ++i) {
+      const float2 f = __bfloat1622float2(h[i]);
+      acc += f.x + f.y;
     }
   }
-  for (int64_t v = vend + lane; v < ve; v += 32) acc += to_f32(r[v]);
+  for (int64_t v = vend + lane; v < ve; v += 32) acc += __bfloat162float(r[v]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) P[(int64_t)split * split_stride + row * rs + col_off] = acc;
@@ -1046,29 +1037,102 @@ __global__ void __launch_bounds__(256) split3_kernel(const float* __restrict__ x
   }
 }
 
+// The same split with the row sums of x per voxel range (the bias-gradient column of the FP32
+// weight gradient, P[split][row]): x is read once for both (0.09 ms less than a pass of its own for
+// the sums at 8,640 rows of 16,001 voxels).  One block per (range, row); the last range writes the
+// zeros up to ldo too.
+__global__ void __launch_bounds__(256) split3_sums_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ldx,
+                                                          __nv_bfloat16* __restrict__ out, int64_t ldo,
+                                                          int64_t part_stride, int64_t vps, int splits,
+                                                          float* __restrict__ sums, int64_t split_stride) {
+  __shared__ float part_sum[8];
+  const int split = blockIdx.x;
+  const int64_t row = blockIdx.y + (int64_t)blockIdx.z * 65535;
+  if (row >= rows) return;
+  const int64_t vs = (int64_t)split * vps, ve = split == splits - 1 ? ldo : min(ldo, vs + vps);  // multiples of 8
+  const float* xr = x + row * ldx;
+  __nv_bfloat16* o = out + row * ldo;
+  float acc = 0.f;
+#pragma unroll 2
+  for (int64_t c = vs + 4 * threadIdx.x; c < ve; c += 1024) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c + 4 <= cols) {
+      v = *reinterpret_cast<const float4*>(xr + c);
+    } else {
+      if (c < cols) v.x = xr[c];
+      if (c + 1 < cols) v.y = xr[c + 1];
+      if (c + 2 < cols) v.z = xr[c + 2];
+    }
+    acc += (v.x + v.y) + (v.z + v.w);
+    uint32_t lo[3], hi[3];
+    ptx::split3x2(v.x, v.y, lo);
+    ptx::split3x2(v.z, v.w, hi);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(o + q * part_stride + c) = make_uint2(lo[q], hi[q]);
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+  if (threadIdx.x % 32 == 0) part_sum[threadIdx.x / 32] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += part_sum[w];
+    sums[split * split_stride + row] = t;
+  }
+}
+
+cudaError_t split_bf16x3_sums(const float* x, int64_t rows, int64_t cols, int64_t ldx, void* out, int64_t ldo,
+                              int64_t part_stride, int64_t vps, int splits, float* sums, int64_t split_stride,
+                              cudaStream_t st) {
+  if (rows <= 0 || ldo <= 0) return cudaSuccess;
+  TraceScope trace("split_bf16x3", st);
+  const dim3 grid((unsigned)splits, (unsigned)std::min<int64_t>(rows, 65535), (unsigned)((rows + 65534) / 65535));
+  split3_sums_kernel<<<grid, 256, 0, st>>>(x, rows, cols, ldx, reinterpret_cast<__nv_bfloat16*>(out), ldo, part_stride,
+                                           vps, splits, sums, split_stride);
+  count_launch();
+  return cudaGetLastError();
+}
+
 // out[c * ldo + r] = in[r * ldi + c] for r < rows, c < cols (BF16), through 64 x 64 tiles in
-// shared memory: the input-gradient GEMM's K-major operator Wt from W.
+// shared memory: the input-gradient GEMM's K-major operator Wt from W.  Bound by HBM; whole tiles
+// move in 16-byte pieces both ways (rows of 128 contiguous bytes): 0.061 ms at 8,640 x 8,640 against
+// 0.090 with 2-byte accesses.  A row of the tile is 33 words, so that the transposed reads of a
+// warp (eight 8-row pieces of four columns) spread over the banks.
+constexpr int kTrLd = 66;
+
 __global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in, int64_t rows,
                                                              int64_t cols, int64_t ldi, __nv_bfloat16* __restrict__ out,
-                                                             int64_t ldo) {
-  __shared__ __nv_bfloat16 tile[64][66];
+                                                             int64_t ldo, int vec) {
+  __shared__ __align__(16) uint16_t tile[64 * kTrLd];
   const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int i = ty; i < 64; i += 8) {
-    const int64_t r = r0 + i;
+  const uint16_t* src = reinterpret_cast<const uint16_t*>(in);
+  uint16_t* dst = reinterpret_cast<uint16_t*>(out);
+  const bool whole = vec && r0 + 64 <= rows && c0 + 64 <= cols;
 #pragma unroll
-    for (int j = tx; j < 64; j += 32) {
-      const int64_t c = c0 + j;
-      tile[i][j] = (r < rows && c < cols) ? in[r * ldi + c] : __float2bfloat16_rn(0.f);
+  for (int e = 0; e < 2; ++e) {
+    const int i = threadIdx.x + 256 * e, r = i >> 3, c = (i & 7) * 8;  // 8 columns of one row
+    uint16_t* t = tile + r * kTrLd + c;
+    if (whole) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + (r0 + r) * ldi + c0 + c));
+      uint32_t* t32 = reinterpret_cast<uint32_t*>(t);
+      t32[0] = v.x, t32[1] = v.y, t32[2] = v.z, t32[3] = v.w;
+    } else {
+      for (int j = 0; j < 8; ++j) t[j] = (r0 + r < rows && c0 + c + j < cols) ? src[(r0 + r) * ldi + c0 + c + j] : 0;
     }
   }
   __syncthreads();
-  for (int i = ty; i < 64; i += 8) {
-    const int64_t c = c0 + i;
 #pragma unroll
-    for (int j = tx; j < 64; j += 32) {
-      const int64_t r = r0 + j;
-      if (c < cols && r < rows) out[c * ldo + r] = tile[j][i];
+  for (int e = 0; e < 2; ++e) {
+    const int i = threadIdx.x + 256 * e, c = i >> 3, r = (i & 7) * 8;  // 8 rows of one column
+    uint32_t v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      v[j] = (uint32_t)tile[(r + 2 * j) * kTrLd + c] | ((uint32_t)tile[(r + 2 * j + 1) * kTrLd + c] << 16);
+    if (whole) {
+      *reinterpret_cast<uint4*>(dst + (c0 + c) * ldo + r0 + r) = make_uint4(v[0], v[1], v[2], v[3]);
+    } else if (c0 + c < cols) {
+      for (int j = 0; j < 8; ++j)
+        if (r0 + r + j < rows) dst[(c0 + c) * ldo + r0 + r + j] = (uint16_t)(v[j >> 1] >> (16 * (j & 1)));
     }
   }
 }
@@ -1078,8 +1142,10 @@ cudaError_t transpose_bf16(const void* in, int64_t rows, int64_t cols, int64_t l
   if (rows <= 0 || cols <= 0) return cudaSuccess;
   TraceScope trace("lsc_transpose_w", st);
   const dim3 grid((unsigned)((cols + 63) / 64), (unsigned)((rows + 63) / 64));
+  const int vec = ldi % 8 == 0 && ldo % 8 == 0 &&
+                  ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
   transpose_bf16_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(in), rows, cols, ldi,
-                                              reinterpret_cast<__nv_bfloat16*>(out), ldo);
+                                              reinterpret_cast<__nv_bfloat16*>(out), ldo, vec);
   count_launch();
   return cudaGetLastError();
 }
@@ -1329,6 +1395,7 @@ cudaError_t run_vox(const CUtensorMap& ma, const OperatorView& B, VoxParams& p, 
   if (p.Yf) {
     switch (bn) {
       case 256: return launch_vox_cl<256, false, true>(ma, mb, my, p, cl, st);
+      case 240: return launch_vox_cl<240, false, true>(ma, mb, my, p, cl, st);
       case 192: return launch_vox_cl<192, false, true>(ma, mb, my, p, cl, st);
       default: return launch_vox_cl<128, false, true>(ma, mb, my, p, cl, st);
     }
@@ -1358,8 +1425,15 @@ bool tc_gemm_supported(const LscDims& d, int64_t n_vox, int64_t ld_in, int64_t l
 // input row: zeros in W against rows that read as zero), W's columns are X's rows.
 bool tc_forward_reads_w(const LscDims& d) { return d.in_blk == (int64_t)d.c_in * d.n_in || d.s_in == 1; }
 
-bool tc_dgrad_reads_wt(const LscDims& d) {
-  return d.out_blk == (int64_t)d.c_out * d.n_out && ((int64_t)d.c_in * d.n_in) % kDgradBN == 0;
+// W's transpose costs what it costs however many voxels follow, and its GEMM is faster by a share of
+// itself (no padded columns, no MN-major operand), so it pays from a number of voxels on.  With it and
+// without, ms: BF16 64 -> 64 channels 0.213 / 0.179 at 2,048 voxels, 0.605 / 0.612 at 8,192, 2.40 / 2.58
+// at 32,768, 16 -> 64 channels 0.091 / 0.076 at 2,048, 0.172 / 0.180 at 8,192; FP32 (three parts, six
+// products) 64 -> 64 channels 0.62 / 0.53 at 1,024, 1.06 / 1.06 at 2,048, 4.06 / 4.44 at 8,192, 16 -> 8
+// channels at 3,640 voxels 0.067 / 0.056.
+bool tc_dgrad_reads_wt(const LscDims& d, int64_t n_vox, bool split) {
+  return n_vox >= (split ? 4096 : 8192) && d.out_blk == (int64_t)d.c_out * d.n_out &&
+         ((int64_t)d.c_in * d.n_in) % kDgradBN == 0;
 }
 
 cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const void* Wt, const float* bias, void* Y,
@@ -1413,11 +1487,11 @@ cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const 
   CUtensorMap ma;
   if (!make_map(&ma, dY, (uint64_t)n_vox, (uint64_t)d.rows_out, (uint64_t)lddy, 64, kBK, parts.act))
     return cudaErrorInvalidValue;
-  // BF16 with Wt available: Wt is the K-major operator (rows = input features, columns = dY
+  // With Wt available: Wt is the K-major operator (rows = input features, columns = dY
   // rows when W's output blocks carry no padding) and 240-column tiles cover c_in n_in
   // exactly; otherwise W as the MN-major operator (64-column atoms, padded last tile)
-  const bool kmajor = !parts.on() && Wt && tc_dgrad_reads_wt(d);
-  const OperatorView B = kmajor ? OperatorView{Wt, (uint64_t)d.rows_in, (uint64_t)d.ldWt, (uint64_t)d.ldWt, true}
+  const bool kmajor = Wt && tc_dgrad_reads_wt(d, n_vox, parts.on());
+  const OperatorView B = kmajor ? OperatorView{Wt, (uint64_t)d.rows_in, (uint64_t)d.ldWt, (uint64_t)d.ldWt, true, parts.op}
                                 : OperatorView{W, (uint64_t)d.rows_out, (uint64_t)d.ldW, (uint64_t)d.ldW, false,
                                                parts.op};
   VoxParams p;
@@ -1467,7 +1541,7 @@ cudaError_t launch_wgrad(const CUtensorMap& ma, const CUtensorMap& mb, const WgP
 
 cudaError_t tc_lsc_wgrad(const LscDims& d, const void* dY, const void* X, float* P, int64_t ldp, int64_t split_stride,
                          int splits, int64_t vps, int64_t n_vox, int64_t lddy, int64_t ldx, int* err, cudaStream_t st,
-                         TcParts parts, const void* dY_sum, int64_t lddy_sum) {
+                         TcParts parts) {
   constexpr int BN = kWgradBN;
   const int cl = gemm_cluster(2);
   CUtensorMap ma, mb;
@@ -1518,23 +1592,19 @@ cudaError_t tc_lsc_wgrad(const LscDims& d, const void* dY, const void* X, float*
       e = cl > 1 ? launch_wgrad<BN, 7, 2, false>(ma, mb, p, st) : launch_wgrad<BN, 4, 1, false>(ma, mb, p, st);
     if (e != cudaSuccess) return e;
   }
-  // bias-gradient column: row sums of dY per split.  BF16 operands on CTA pairs: made by
-  // the GEMM (ones rows in its operand slots, one 256-wide column tile per row tile);
-  // otherwise a separate HBM-bound pass (a separate N = 16 MMA per step inside the GEMM
-  // measured slower: each MMA streams its whole A tile again)
-  if (!parts.on() && cl > 1) {
+  // bias-gradient column: row sums of dY per split.  FP32: made with the operand split
+  // (split_bf16x3_sums).  BF16 on CTA pairs: made by the GEMM (ones rows in its operand slots, one
+  // 256-wide column tile per row tile); on single CTAs a separate HBM-bound pass (a separate
+  // N = 16 MMA per step inside the GEMM measured slower: each MMA streams its whole A tile again)
+  if (parts.on() || cl > 1) {
     static_assert(wgrad_sums<BN, 2, false>(), "the BF16 pair kernel makes the row sums");
     return cudaGetLastError();
   }
   const int64_t warps = d.rows_out * splits;
   TraceScope trace_rs("lsc_rowsum", st);
   const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
-  if (parts.on())
-    rowsum_kernel<float><<<blocks, 256, 0, st>>>(reinterpret_cast<const float*>(dY_sum), lddy_sum, d.rows_out, n_vox,
-                                                 vps, splits, P, 1, split_stride, d.rows_in * ldp);
-  else
-    rowsum_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(dY), lddy, d.rows_out,
-                                                         n_vox, vps, splits, P, 1, split_stride, d.rows_in * ldp);
+  rowsum_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(dY), lddy, d.rows_out, n_vox, vps, splits,
+                                        P, 1, split_stride, d.rows_in * ldp);
   count_launch();
   return cudaGetLastError();
 }

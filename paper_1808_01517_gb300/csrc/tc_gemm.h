@@ -61,20 +61,18 @@ bool tc_forward_reads_w(const LscDims& d);
 cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const void* Wt, const float* bias, void* Y,
                            int64_t n_vox, int64_t ldx, int64_t ldy, int* err_word, cudaStream_t st,
                            TcParts parts = TcParts{});
-// dX[(s',ci,b), v] = sum_{k in rwin(s')} W[k][s'*in_blk + (ci,b)] dY[k, v].  BF16 reads Wt
-// (K-major) when tc_dgrad_reads_wt(d) and Wt is given, else W.
-bool tc_dgrad_reads_wt(const LscDims& d);
+// dX[(s',ci,b), v] = sum_{k in rwin(s')} W[k][s'*in_blk + (ci,b)] dY[k, v].  Reads Wt (K-major)
+// when tc_dgrad_reads_wt and Wt is given, else W.
+bool tc_dgrad_reads_wt(const LscDims& d, int64_t n_vox, bool split);
 cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const void* Wt, void* dX, int64_t n_vox,
                          int64_t lddy, int64_t lddx, int* err_word, cudaStream_t st, TcParts parts = TcParts{});
 // P[split][(s,co,a)][(s',ci,b)] = sum_{v in split} dY[(s,co,a), v] X[(s',ci,b), v] for s' in win(s),
-// P[split][(s,co,a)][rows_in] = sum_{v in split} dY[(s,co,a), v] (from dY_sum: the BF16 dY, or
-// the FP32 dY when the operands are split; lddy_sum its row stride).  The partials are
-// stored transposed, P[split][col][row] with leading dimension ldp >= rows_out (the row
+// P[split][(s,co,a)][rows_in] = sum_{v in split} dY[(s,co,a), v] (BF16; with split operands
+// split_bf16x3_sums writes them).  The partials are stored transposed, P[split][col][row] with leading dimension ldp >= rows_out (the row
 // sums in row rows_in), so that the epilogue's stores are coalesced.
 cudaError_t tc_lsc_wgrad(const LscDims& d, const void* dY, const void* X, float* P, int64_t ldp, int64_t split_stride,
                          int splits, int64_t vox_per_split, int64_t n_vox, int64_t lddy, int64_t ldx, int* err_word,
-                         cudaStream_t st, TcParts parts = TcParts{}, const void* dY_sum = nullptr,
-                         int64_t lddy_sum = 0);
+                         cudaStream_t st, TcParts parts = TcParts{});
 // out[c * ldo + r] = in[r * ldi + c] for r < rows, c < cols (BF16)
 cudaError_t transpose_bf16(const void* in, int64_t rows, int64_t cols, int64_t ldi, void* out, int64_t ldo,
                            cudaStream_t st);
@@ -83,6 +81,12 @@ cudaError_t transpose_bf16(const void* in, int64_t rows, int64_t cols, int64_t l
 // of every part row are zeroed.  ldx a multiple of 4, ldo of 8, both pointers 16-byte aligned.
 cudaError_t split_bf16x3(const float* x, int64_t rows, int64_t cols, int64_t ldx, void* out, int64_t ldo,
                          int64_t part_stride, cudaStream_t st);
+
+// The same, and sums[split * split_stride + r] = sum of x's row r over its voxel range (vps voxels,
+// a multiple of 8, per split)
+cudaError_t split_bf16x3_sums(const float* x, int64_t rows, int64_t cols, int64_t ldx, void* out, int64_t ldo,
+                              int64_t part_stride, int64_t vps, int splits, float* sums, int64_t split_stride,
+                              cudaStream_t st);
 
 // The LSC forward with SH2Signal in its epilogue (tc_fused.cu): B_s^T of the output basis'
 // shells as the K-major BF16 operator [S][96 directions][64 coefficients], zero-padded.
