@@ -308,6 +308,15 @@ delimit_status delimit_lsc_forward(const delimit_lsc_geometry* geom, const void*
                                    int64_t ld_in, int64_t ld_out, delimit_dtype act_t, unsigned flags,
                                    void* workspace, size_t ws_bytes, void* stream);
 
+/* delimit_lsc_forward with a leaky ReLU on its output (slope as delimit_leaky_relu, on the value
+ * as delimit_lsc_forward stores it): the same result as the two calls one after the other.
+ * BF16 on the tensor cores applies it in the GEMM's epilogue, the other paths as a pass over
+ * sh_out.  Arguments and errors otherwise as delimit_lsc_forward. */
+delimit_status delimit_lsc_forward_leaky(const delimit_lsc_geometry* geom, const void* sh_in, const float* w,
+                                         const float* b, void* sh_out, float slope, int64_t n_vox, int c_in,
+                                         int c_out, int64_t ld_in, int64_t ld_out, delimit_dtype act_t,
+                                         unsigned flags, void* workspace, size_t ws_bytes, void* stream);
+
 /* The LSC forward followed by SH2Signal on the output basis' directions, in one kernel
  * (Sec. 2.3: the paper's LSC example pipes SH -> LSC -> SH2Signal; Sec. 2.2 for
  * SH2Signal):
@@ -350,6 +359,17 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* geom, const void
                                     const void* d_out, void* d_in, float* dw, float* db, int64_t n_vox,
                                     int c_in, int c_out, int64_t ld_in, int64_t ld_out, delimit_dtype act_t,
                                     unsigned flags, void* workspace, size_t ws_bytes, void* stream);
+
+/* delimit_lsc_backward where sh_in is the output of a leaky ReLU with this slope: d_in is the
+ * gradient of that leaky ReLU's input, i.e. delimit_leaky_relu_backward of sh_in and the d_in
+ * of delimit_lsc_backward (the same result; in the GEMM's epilogue for BF16 on the tensor
+ * cores).  sh_in is needed for d_in here.  Arguments and errors otherwise as
+ * delimit_lsc_backward. */
+delimit_status delimit_lsc_backward_leaky(const delimit_lsc_geometry* geom, const void* sh_in, const float* w,
+                                          const void* d_out, void* d_in, float* dw, float* db, float slope,
+                                          int64_t n_vox, int c_in, int c_out, int64_t ld_in, int64_t ld_out,
+                                          delimit_dtype act_t, unsigned flags, void* workspace, size_t ws_bytes,
+                                          void* stream);
 
 /* ------------------------------------------------------------------------ */
 /* Helpers of the learned network and whole-volume inference (no counterpart */

@@ -73,6 +73,10 @@ SIGNATURES = {
                                       _vp, C.c_size_t, _vp]),
     "delimit_lsc_backward": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _i64, C.c_int, C.c_int, _i64, _i64,
                                        C.c_int, C.c_uint, _vp, C.c_size_t, _vp]),
+    "delimit_lsc_forward_leaky": (C.c_int, [_vp, _vp, _vp, _vp, _vp, C.c_float, _i64, C.c_int, C.c_int, _i64, _i64,
+                                            C.c_int, C.c_uint, _vp, C.c_size_t, _vp]),
+    "delimit_lsc_backward_leaky": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, C.c_float, _i64, C.c_int, C.c_int,
+                                             _i64, _i64, C.c_int, C.c_uint, _vp, C.c_size_t, _vp]),
     "delimit_lsc_forward_sh2signal": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _i64, C.c_int, C.c_int, _i64, _i64,
                                                 C.c_int, C.c_uint, _vp, C.c_size_t, _vp]),
     "delimit_lsc_forward_sh2signal_supported": (C.c_int, [_vp, _i64, C.c_int, C.c_int, C.c_int]),

@@ -785,6 +785,17 @@ size_t delimit_lsc_workspace_size(const delimit_lsc_geometry* g, int64_t n_vox, 
   return backward ? p.total_bwd : p.total_fwd;
 }
 
+// leaky ReLU over an output in place (rows in slices of what the elementwise call takes)
+static delimit_status leaky_pass(void* y, const float* slope, int64_t rows, int64_t n_vox, int64_t ld, delimit_dtype t,
+                                 void* stream) {
+  for (int64_t r = 0; slope && r < rows; r += 65535) {
+    char* p = static_cast<char*>(y) + r * ld * elem_size(t);
+    const delimit_status st = delimit_leaky_relu(p, p, std::min<int64_t>(65535, rows - r), n_vox, ld, ld, *slope, t, stream);
+    if (st != DELIMIT_OK) return st;
+  }
+  return DELIMIT_OK;
+}
+
 static delimit_status lsc_common_checks(const delimit_lsc_geometry* g, int64_t n_vox, int c_in, int c_out,
                                         delimit_dtype t, void* ws, size_t ws_bytes, bool bwd, LscPlan& p) {
   if (!g) return fail(DELIMIT_ERR_INVALID_ARG, "geometry is NULL");
@@ -803,9 +814,12 @@ static delimit_status lsc_common_checks(const delimit_lsc_geometry* g, int64_t n
   return DELIMIT_OK;
 }
 
-delimit_status delimit_lsc_forward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const float* b,
-                                   void* sh_out, int64_t n_vox, int c_in, int c_out, int64_t ld_in, int64_t ld_out,
-                                   delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes, void* stream) {
+// slope: NULL, or the leaky ReLU applied to sh_out (in the GEMM's epilogue where BF16 runs on the
+// tensor cores, else as a pass over it)
+static delimit_status lsc_forward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const float* b,
+                                  void* sh_out, const float* slope, int64_t n_vox, int c_in, int c_out, int64_t ld_in,
+                                  int64_t ld_out, delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes,
+                                  void* stream) {
   LscPlan p;
   delimit_status st = lsc_common_checks(g, n_vox, c_in, c_out, act_t, ws, ws_bytes, false, p);
   if (st != DELIMIT_OK) return st;
@@ -837,10 +851,13 @@ delimit_status delimit_lsc_forward(const delimit_lsc_geometry* g, const void* sh
     e = tc_lsc_forward(d, X3, base + p.off_W3, base + p.off_Wt3, bias, sh_out, n_vox, p.ld3, ld_out, g->err_word, cs,
                        parts);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core FP32 LSC forward launch");
-    return DELIMIT_OK;
+    return leaky_pass(sh_out, slope, d.rows_out, n_vox, ld_out, act_t, stream);
   }
   if (tc && act_t == DELIMIT_BF16) {
-    e = tc_lsc_forward(d, sh_in, W, Wt, bias, sh_out, n_vox, ld_in, ld_out, g->err_word, cs);
+    TcLeaky act;
+    act.on = slope != nullptr;
+    act.slope = slope ? *slope : 0.f;
+    e = tc_lsc_forward(d, sh_in, W, Wt, bias, sh_out, n_vox, ld_in, ld_out, g->err_word, cs, TcParts{}, act);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core LSC forward launch");
     return DELIMIT_OK;
   }
@@ -867,7 +884,22 @@ delimit_status delimit_lsc_forward(const delimit_lsc_geometry* g, const void* sh
   a.n_vox = n_vox;
   e = launch_row_gemm_simt(a, d.s_out, per_out, int(act_t), cs);
   if (e != cudaSuccess) return cuda_fail(e, "LSC forward launch");
-  return DELIMIT_OK;
+  return leaky_pass(sh_out, slope, d.rows_out, n_vox, ld_out, act_t, stream);
+}
+
+delimit_status delimit_lsc_forward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const float* b,
+                                   void* sh_out, int64_t n_vox, int c_in, int c_out, int64_t ld_in, int64_t ld_out,
+                                   delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes, void* stream) {
+  return lsc_forward(g, sh_in, w, b, sh_out, nullptr, n_vox, c_in, c_out, ld_in, ld_out, act_t, flags, ws, ws_bytes,
+                     stream);
+}
+
+delimit_status delimit_lsc_forward_leaky(const delimit_lsc_geometry* g, const void* sh_in, const float* w,
+                                         const float* b, void* sh_out, float slope, int64_t n_vox, int c_in, int c_out,
+                                         int64_t ld_in, int64_t ld_out, delimit_dtype act_t, unsigned flags, void* ws,
+                                         size_t ws_bytes, void* stream) {
+  return lsc_forward(g, sh_in, w, b, sh_out, &slope, n_vox, c_in, c_out, ld_in, ld_out, act_t, flags, ws, ws_bytes,
+                     stream);
 }
 
 delimit_status delimit_lsc_forward_sh2signal_supported(const delimit_lsc_geometry* g, int64_t n_vox, int c_in,
@@ -913,10 +945,12 @@ delimit_status delimit_lsc_forward_sh2signal(const delimit_lsc_geometry* g, cons
   return DELIMIT_OK;
 }
 
-delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const void* d_out,
-                                    void* d_in, float* dw, float* db, int64_t n_vox, int c_in, int c_out, int64_t ld_in,
-                                    int64_t ld_out, delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes,
-                                    void* stream) {
+// slope: NULL, or sh_in is the output of a leaky ReLU with that slope and d_in the gradient of its
+// input (in the GEMM's epilogue where BF16 runs on the tensor cores, else as a pass over d_in)
+static delimit_status lsc_backward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const void* d_out,
+                                   void* d_in, float* dw, float* db, const float* slope, int64_t n_vox, int c_in,
+                                   int c_out, int64_t ld_in, int64_t ld_out, delimit_dtype act_t, unsigned flags,
+                                   void* ws, size_t ws_bytes, void* stream) {
   LscPlan p;
   delimit_status st = lsc_common_checks(g, n_vox, c_in, c_out, act_t, ws, ws_bytes, true, p);
   if (st != DELIMIT_OK) return st;
@@ -934,7 +968,7 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* s
     return DELIMIT_OK;
   }
   if ((st = check_act(d_out, ld_out, n_vox, act_t, "d_out")) != DELIMIT_OK) return st;
-  if (dw || db)
+  if (dw || db || (d_in && slope))
     if ((st = check_act(sh_in, ld_in, n_vox, act_t, "sh_in")) != DELIMIT_OK) return st;
   if (d_in) {
     if ((st = check_act(d_in, ld_in, n_vox, act_t, "d_in")) != DELIMIT_OK) return st;
@@ -992,7 +1026,12 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* s
         e = transpose_bf16(W, d.rows_out, d.ldW, d.ldW, Wt, d.ldWt, cs);
         if (e != cudaSuccess) return cuda_fail(e, "operator transpose launch");
       }
-      e = tc_lsc_dgrad(d, d_out, W, wt_k ? Wt : nullptr, d_in, n_vox, ld_out, ld_in, g->err_word, cs);
+      TcLeaky act;
+      act.on = slope != nullptr;
+      act.slope = slope ? *slope : 0.f;
+      act.mask = sh_in;
+      act.ldmask = ld_in;
+      e = tc_lsc_dgrad(d, d_out, W, wt_k ? Wt : nullptr, d_in, n_vox, ld_out, ld_in, g->err_word, cs, TcParts{}, act);
       if (e != cudaSuccess) return cuda_fail(e, "tensor-core LSC input-gradient launch");
     } else {
       if ((st = cuda_core_path("LSC input gradient")) != DELIMIT_OK) return st;
@@ -1017,6 +1056,15 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* s
       a.n_vox = n_vox;
       e = launch_row_gemm_simt(a, d.s_in, per_in, int(act_t), cs);
       if (e != cudaSuccess) return cuda_fail(e, "LSC input-gradient launch");
+    }
+    const size_t es = elem_size(act_t);
+    const bool in_epilogue = act_t == DELIMIT_BF16 && all_fed && tc;
+    for (int64_t r = 0; slope && !in_epilogue && r < d.rows_in; r += 65535) {
+      char* dp = static_cast<char*>(d_in) + r * ld_in * es;
+      st = delimit_leaky_relu_backward(static_cast<const char*>(sh_in) + r * ld_in * es, dp, dp,
+                                       std::min<int64_t>(65535, d.rows_in - r), n_vox, ld_in, ld_in, ld_in, *slope, act_t,
+                                       stream);
+      if (st != DELIMIT_OK) return st;
     }
   }
   if (dw || db) {
@@ -1083,6 +1131,22 @@ delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* s
     if (e != cudaSuccess) return cuda_fail(e, "dw/db reduction launch");
   }
   return DELIMIT_OK;
+}
+
+delimit_status delimit_lsc_backward(const delimit_lsc_geometry* g, const void* sh_in, const float* w, const void* d_out,
+                                    void* d_in, float* dw, float* db, int64_t n_vox, int c_in, int c_out, int64_t ld_in,
+                                    int64_t ld_out, delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes,
+                                    void* stream) {
+  return lsc_backward(g, sh_in, w, d_out, d_in, dw, db, nullptr, n_vox, c_in, c_out, ld_in, ld_out, act_t, flags, ws,
+                      ws_bytes, stream);
+}
+
+delimit_status delimit_lsc_backward_leaky(const delimit_lsc_geometry* g, const void* sh_in, const float* w,
+                                          const void* d_out, void* d_in, float* dw, float* db, float slope,
+                                          int64_t n_vox, int c_in, int c_out, int64_t ld_in, int64_t ld_out,
+                                          delimit_dtype act_t, unsigned flags, void* ws, size_t ws_bytes, void* stream) {
+  return lsc_backward(g, sh_in, w, d_out, d_in, dw, db, &slope, n_vox, c_in, c_out, ld_in, ld_out, act_t, flags, ws,
+                      ws_bytes, stream);
 }
 
 delimit_status delimit_selftest_wait_timeout(void* stream) {

@@ -110,8 +110,22 @@ struct VoxParams {
   __nv_bfloat16* Y;
   float* Yf;  // FP32 output (direct stores) in place of Y
   const float* bias;
+  // leaky ReLU in the epilogue (BF16 outputs), on the value rounded to BF16 as a pass of its own
+  // would read it: the output scaled by slope where it is not positive or, for the adjoint, where
+  // `mask`, an activation laid out like Y, is not
+  int leaky;  // which instantiation runs
+  float slope;
+  const __nv_bfloat16* mask;  // null: the output itself
+  int64_t ldmask;
   int* err;
 };
+
+// a pair of values, each scaled by slope where its mask is not positive
+__device__ __forceinline__ uint32_t leaky_bf16x2(uint32_t x, uint32_t mask, float slope) {
+  const float lo = __uint_as_float(x << 16), hi = __uint_as_float(x & 0xFFFF0000u);
+  return ptx::pack_bf16x2f(__uint_as_float(mask << 16) > 0.f ? lo : slope * lo,
+                           __uint_as_float(mask & 0xFFFF0000u) > 0.f ? hi : slope * hi);
+}
 
 // Tile order: kVoxGroup voxel tiles are walked together, operator tile by operator tile (voxel tile
 // fastest), then the next group; persistent clusters take tiles round-robin.  The 76 tiles in flight
@@ -151,7 +165,10 @@ __device__ __forceinline__ void vox_decode(const VoxParams& p, int64_t t, int& g
 // each CTA's TMEM receives its own 128 voxels x BN accumulator, drained by its
 // own epilogue, which hands the buffer back on the even CTA's barrier.
 // p.total_tiles counts cluster tiles (voxel-tile pairs x operator tiles).
-template <int BN, int STAGES, bool STAGED, int PASSES, int CL, bool SPLIT>
+// LEAKY: the leaky ReLU or its adjoint in the epilogue.  A template, as the code alone, not taken,
+// cost the plain layers up to a fifth of a small call's time (4 -> 64 channels at 1,431 voxels 16 -> 20
+// us, the input gradient of 8 -> 8 at 4,456 voxels 30 -> 36).
+template <int BN, int STAGES, bool STAGED, int PASSES, int CL, bool SPLIT, bool LEAKY>
 __global__ void __launch_bounds__(kThreads, 1)
     vox_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ CUtensorMap mapY, const __grid_constant__ VoxParams p) {
@@ -448,10 +465,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int lb = 0; lb < 2; ++lb) {
                   const uint32_t* r0 = rv[u][lb][0];
                   const uint32_t* r1 = rv[u][lb][1];
-                  const uint32_t m0 = pack_bf16x2f(__uint_as_float(r0[0]) + b[0], __uint_as_float(r0[1]) + b[1]);
-                  const uint32_t m1 = pack_bf16x2f(__uint_as_float(r0[2]) + b[0], __uint_as_float(r0[3]) + b[1]);
-                  const uint32_t m2 = pack_bf16x2f(__uint_as_float(r1[0]) + b[2], __uint_as_float(r1[1]) + b[3]);
-                  const uint32_t m3 = pack_bf16x2f(__uint_as_float(r1[2]) + b[2], __uint_as_float(r1[3]) + b[3]);
+                  uint32_t m0 = pack_bf16x2f(__uint_as_float(r0[0]) + b[0], __uint_as_float(r0[1]) + b[1]);
+                  uint32_t m1 = pack_bf16x2f(__uint_as_float(r0[2]) + b[0], __uint_as_float(r0[3]) + b[1]);
+                  uint32_t m2 = pack_bf16x2f(__uint_as_float(r1[0]) + b[2], __uint_as_float(r1[1]) + b[3]);
+                  uint32_t m3 = pack_bf16x2f(__uint_as_float(r1[2]) + b[2], __uint_as_float(r1[3]) + b[3]);
+                  if (LEAKY && !p.mask) {
+                    m0 = leaky_bf16x2(m0, m0, p.slope);
+                    m1 = leaky_bf16x2(m1, m1, p.slope);
+                    m2 = leaky_bf16x2(m2, m2, p.slope);
+                    m3 = leaky_bf16x2(m3, m3, p.slope);
+                  }
                   const int c = (c0 - cbeg) + ((mm >> 1) << 3) + rr, vc = vq + 2 * lb + (mm & 1);
                   stmatrix_x4_trans(stg_h + (uint32_t)(c * 128 + ((vc ^ (c & 7)) << 4)), m0, m1, m2, m3);
                 }
@@ -473,23 +496,68 @@ __global__ void __launch_bounds__(kThreads, 1)
           // copy-out: 16-byte chunks (8 voxels) of the tile, a warp per 4 rows x 8 chunks, i.e.
           // four 128-byte row segments of Y per store instruction (conflict-free 128-bit
           // shared loads); rows past the group's N and voxels past n_vox are not written
-          {
-            const int et = threadIdx.x - 64;
+          const int et = threadIdx.x - 64;
+          constexpr int NE = 2 * HB * 8 / (32 * kEpiWarps);  // chunks per thread
+          auto chunk = [&](int e, int& col, int64_t& v0) -> const uint8_t* {  // its staging address, row and first voxel
+            const int i = et + 32 * kEpiWarps * e, j = i & 7, rowh = i >> 3;
+            const int hh = rowh >= HB ? 1 : 0, c = rowh - hh * HB;
+            col = nt * BN + cbeg + c;
+            v0 = (int64_t)mt * 128 + 64 * hh + 8 * j;
+            return stg_ptr + (hh * HB + c) * 128 + ((j ^ (c & 7)) << 4);
+          };
+          if (!LEAKY || !p.mask) {
 #pragma unroll 4
-            for (int e = 0; e < 2 * HB * 8 / (32 * kEpiWarps); ++e) {
-              const int i = et + 32 * kEpiWarps * e, j = i & 7, rowh = i >> 3;
-              const int hh = rowh >= HB ? 1 : 0, c = rowh - hh * HB;
-              const int col = nt * BN + cbeg + c;
-              const int64_t v0 = (int64_t)mt * 128 + 64 * hh + 8 * j;
+            for (int e = 0; e < NE; ++e) {
+              int col;
+              int64_t v0;
+              const uint8_t* src = chunk(e, col, v0);
               if (col >= G.N || v0 >= p.n_vox) continue;
-              const uint4 val =
-                  *reinterpret_cast<const uint4*>(stg_ptr + (hh * HB + c) * 128 + ((j ^ (c & 7)) << 4));
+              const uint4 val = *reinterpret_cast<const uint4*>(src);
               __nv_bfloat16* dst = p.Y + (G.y_row0 + col) * p.ldy + v0;
               if (v0 + 8 <= p.n_vox) {
                 __stcs(reinterpret_cast<int4*>(dst), make_int4((int)val.x, (int)val.y, (int)val.z, (int)val.w));
               } else {
                 const __nv_bfloat16* v8 = reinterpret_cast<const __nv_bfloat16*>(&val);
                 for (int k = 0; k < 8 && v0 + k < p.n_vox; ++k) dst[k] = v8[k];
+              }
+            }
+          } else {
+            // with the leaky ReLU's adjoint, all the thread's masks in flight before they are used (64 -> 1
+            // channels at 8,192 voxels 0.112 ms, half of them at a time 0.126, four at a time 0.266)
+            uint4 mv[NE];
+#pragma unroll
+            for (int u = 0; u < NE; ++u) {
+              int col;
+              int64_t v0;
+              chunk(u, col, v0);
+              mv[u] = make_uint4(0u, 0u, 0u, 0u);
+              if (col >= G.N || v0 >= p.n_vox) continue;
+              const __nv_bfloat16* msrc = p.mask + (G.y_row0 + col) * p.ldmask + v0;
+              if (v0 + 8 <= p.n_vox) {
+                mv[u] = __ldg(reinterpret_cast<const uint4*>(msrc));
+              } else {
+                uint32_t m2[4] = {0u, 0u, 0u, 0u};
+                for (int k = 0; k < 8; ++k)
+                  if (v0 + k < p.n_vox) m2[k >> 1] |= (uint32_t)__bfloat16_as_ushort(msrc[k]) << (16 * (k & 1));
+                mv[u] = make_uint4(m2[0], m2[1], m2[2], m2[3]);
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < NE; ++u) {
+              int col;
+              int64_t v0;
+              const uint8_t* src = chunk(u, col, v0);
+              if (col >= G.N || v0 >= p.n_vox) continue;
+              const uint4 val = *reinterpret_cast<const uint4*>(src), m = mv[u];
+              const uint32_t o2[4] = {leaky_bf16x2(val.x, m.x, p.slope), leaky_bf16x2(val.y, m.y, p.slope),
+                                      leaky_bf16x2(val.z, m.z, p.slope), leaky_bf16x2(val.w, m.w, p.slope)};
+              __nv_bfloat16* dst = p.Y + (G.y_row0 + col) * p.ldy + v0;
+              if (v0 + 8 <= p.n_vox) {
+                __stcs(reinterpret_cast<uint4*>(dst), make_uint4(o2[0], o2[1], o2[2], o2[3]));
+              } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                  if (v0 + k < p.n_vox) dst[k] = __ushort_as_bfloat16((unsigned short)(o2[k >> 1] >> (16 * (k & 1))));
               }
             }
           }
@@ -529,6 +597,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int c0 = 32 * (k0 + u) + 16 * half;
                 const int nbase = nt * BN + c0;
                 if (c0 < BN && nbase < G.N) {
+                  if constexpr (LEAKY) {  // or its adjoint
+                    __nv_bfloat16 mk[16];
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj)
+                      mk[jj] = p.mask && vok && nbase + jj < G.N ? p.mask[(G.y_row0 + nbase + jj) * p.ldmask + vox]
+                                                                 : __float2bfloat16_rn(0.f);
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj) {
+                      const int w = 16 * (k0 + u) + jj;
+                      const float bv = __shfl_sync(0xffffffffu, breg[(w >> 5) < NBREG ? (w >> 5) : 0], w & 31);
+                      if (nbase + jj < G.N && vok) {
+                        const float v = __bfloat162float(__float2bfloat16_rn(__uint_as_float(rv[u][jj]) + bv));
+                        const float m = p.mask ? __bfloat162float(mk[jj]) : v;
+                        p.Y[(G.y_row0 + nbase + jj) * p.ldy + vox] = __float2bfloat16_rn(m > 0.f ? v : p.slope * v);
+                      }
+                    }
+                    continue;
+                  }
 #pragma unroll
                   for (int jj = 0; jj < 16; ++jj) {
                     const int w = 16 * (k0 + u) + jj;
@@ -1293,13 +1379,13 @@ cudaError_t launch_persistent(void (*kern)(Params...), int64_t tiles, int cl, si
   return e;
 }
 
-template <int BN, bool STAGED, int CL, bool SPLIT>
+template <int BN, bool STAGED, int CL, bool SPLIT, bool LEAKY>
 cudaError_t launch_vox(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& my, const VoxParams& p,
                        cudaStream_t st) {
   constexpr int S = vox_stages<BN, STAGED, CL>();
   const size_t smem =
       smem_bytes<BN, S>(2 * kBoxBytes, (BN / CL) * 128) + (STAGED ? BN / kFwdPasses * 256 : 0) + 16;
-  auto kern = vox_gemm_kernel<BN, S, STAGED, kFwdPasses, CL, SPLIT>;
+  auto kern = vox_gemm_kernel<BN, S, STAGED, kFwdPasses, CL, SPLIT, LEAKY>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_persistent(kern, p.total_tiles, CL, smem, st, ma, mb, my, p);
@@ -1307,7 +1393,7 @@ cudaError_t launch_vox(const CUtensorMap& ma, const CUtensorMap& mb, const CUten
   return cudaGetLastError();
 }
 
-template <int BN, bool STAGED, bool SPLIT = false>
+template <int BN, bool STAGED, bool SPLIT, bool LEAKY>
 cudaError_t launch_vox_cl(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& my, VoxParams& p, int cl,
                           cudaStream_t st) {
   if constexpr ((BN / 2) % 8 == 0) {
@@ -1315,12 +1401,25 @@ cudaError_t launch_vox_cl(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     if (cl > 1 && (p.b_kmajor || (BN / 2) % 64 == 0)) {
       p.m_units = (p.m_tiles + 1) / 2;
       p.total_tiles = (int64_t)p.m_units * p.tiles_per_m;
-      return launch_vox<BN, STAGED, 2, SPLIT>(ma, mb, my, p, st);
+      return launch_vox<BN, STAGED, 2, SPLIT, LEAKY>(ma, mb, my, p, st);
     }
   }
   p.m_units = p.m_tiles;
   p.total_tiles = (int64_t)p.m_tiles * p.tiles_per_m;
-  return launch_vox<BN, STAGED, 1, SPLIT>(ma, mb, my, p, st);
+  return launch_vox<BN, STAGED, 1, SPLIT, LEAKY>(ma, mb, my, p, st);
+}
+
+template <bool STAGED, bool SPLIT, bool LEAKY>
+cudaError_t launch_vox_bn(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& my, VoxParams& p, int bn, int cl,
+                          cudaStream_t st) {
+  switch (bn) {
+    case 256: return launch_vox_cl<256, STAGED, SPLIT, LEAKY>(ma, mb, my, p, cl, st);
+    case 240:
+      if constexpr (!STAGED) return launch_vox_cl<240, STAGED, SPLIT, LEAKY>(ma, mb, my, p, cl, st);
+      return cudaErrorInvalidValue;
+    case 192: return launch_vox_cl<192, STAGED, SPLIT, LEAKY>(ma, mb, my, p, cl, st);
+    default: return launch_vox_cl<128, STAGED, SPLIT, LEAKY>(ma, mb, my, p, cl, st);
+  }
 }
 
 // choose the N tile that wastes the fewest columns over the groups (ties: larger)
@@ -1385,27 +1484,12 @@ cudaError_t run_vox(const CUtensorMap& ma, const OperatorView& B, VoxParams& p, 
   // the staged copy-out writes 16-byte chunks at voxel offsets that are multiples of 8
   bool staged = staged_ok && same_n && (bn <= 192 || cl > 1) && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0 &&
                 ldy % 8 == 0;
-  if (staged) {
-    switch (bn) {
-      case 256: return launch_vox_cl<256, true>(ma, mb, my, p, cl, st);
-      case 192: return launch_vox_cl<192, true>(ma, mb, my, p, cl, st);
-      default: return launch_vox_cl<128, true>(ma, mb, my, p, cl, st);
-    }
-  }
-  if (p.Yf) {
-    switch (bn) {
-      case 256: return launch_vox_cl<256, false, true>(ma, mb, my, p, cl, st);
-      case 240: return launch_vox_cl<240, false, true>(ma, mb, my, p, cl, st);
-      case 192: return launch_vox_cl<192, false, true>(ma, mb, my, p, cl, st);
-      default: return launch_vox_cl<128, false, true>(ma, mb, my, p, cl, st);
-    }
-  }
-  switch (bn) {
-    case 256: return launch_vox_cl<256, false>(ma, mb, my, p, cl, st);
-    case 240: return launch_vox_cl<240, false>(ma, mb, my, p, cl, st);
-    case 192: return launch_vox_cl<192, false>(ma, mb, my, p, cl, st);
-    default: return launch_vox_cl<128, false>(ma, mb, my, p, cl, st);
-  }
+  if (staged)
+    return p.leaky ? launch_vox_bn<true, false, true>(ma, mb, my, p, bn, cl, st)
+                   : launch_vox_bn<true, false, false>(ma, mb, my, p, bn, cl, st);
+  if (p.Yf) return launch_vox_bn<false, true, false>(ma, mb, my, p, bn, cl, st);
+  return p.leaky ? launch_vox_bn<false, false, true>(ma, mb, my, p, bn, cl, st)
+                 : launch_vox_bn<false, false, false>(ma, mb, my, p, bn, cl, st);
 }
 
 }  // namespace
@@ -1437,7 +1521,7 @@ bool tc_dgrad_reads_wt(const LscDims& d, int64_t n_vox, bool split) {
 }
 
 cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const void* Wt, const float* bias, void* Y,
-                           int64_t n_vox, int64_t ldx, int64_t ldy, int* err, cudaStream_t st, TcParts parts) {
+                           int64_t n_vox, int64_t ldx, int64_t ldy, int* err, cudaStream_t st, TcParts parts, TcLeaky act) {
   TraceScope trace(parts.on() ? "lsc_fwd_gemm_f32" : "lsc_fwd_gemm", st);
   CUtensorMap ma;
   if (!make_map(&ma, X, (uint64_t)n_vox, (uint64_t)d.rows_in, (uint64_t)ldx, 64, kBK, parts.act))
@@ -1474,6 +1558,8 @@ cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const
   else
     p.Y = reinterpret_cast<__nv_bfloat16*>(Y);
   p.bias = bias;
+  p.leaky = act.on ? 1 : 0;
+  p.slope = act.slope;
   p.err = err;
   // forward tiles are short in K and wide in output: stage the epilogue through TMA stores
   int bn = pick_bn(Ns, d.s_out);
@@ -1482,7 +1568,7 @@ cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const
 }
 
 cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const void* Wt, void* dX, int64_t n_vox,
-                         int64_t lddy, int64_t lddx, int* err, cudaStream_t st, TcParts parts) {
+                         int64_t lddy, int64_t lddx, int* err, cudaStream_t st, TcParts parts, TcLeaky act) {
   TraceScope trace(parts.on() ? "lsc_dgrad_gemm_f32" : "lsc_dgrad_gemm", st);
   CUtensorMap ma;
   if (!make_map(&ma, dY, (uint64_t)n_vox, (uint64_t)d.rows_out, (uint64_t)lddy, 64, kBK, parts.act))
@@ -1518,6 +1604,10 @@ cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const 
   else
     p.Y = reinterpret_cast<__nv_bfloat16*>(dX);
   p.bias = nullptr;
+  p.leaky = act.on ? 1 : 0;
+  p.mask = act.on ? reinterpret_cast<const __nv_bfloat16*>(act.mask) : nullptr;
+  p.ldmask = act.ldmask;
+  p.slope = act.slope;
   p.err = err;
   const int bn = kmajor ? kDgradBN : pick_bn(Ns, d.s_in);
   // A short K leaves a tile's time to its stores: whole row segments through the staging tile (64 -> 1

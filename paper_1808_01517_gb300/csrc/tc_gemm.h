@@ -53,6 +53,15 @@ struct TcParts {
   int64_t act = 0, op = 0, act2 = 0;  // act2: the weight gradient's second activation (X)
   bool on() const { return act != 0; }
 };
+// Leaky ReLU in a GEMM's epilogue (BF16 outputs): of the forward's output, or, with `mask` (an
+// activation of the input gradient's layout, row stride ldmask), of the input gradient, scaled by
+// slope where the mask is not positive.
+struct TcLeaky {
+  bool on = false;
+  float slope = 0.f;
+  const void* mask = nullptr;
+  int64_t ldmask = 0;
+};
 bool tc_gemm_supported(const LscDims& d, int64_t n_vox, int64_t ld_in, int64_t ld_out);
 // Y[(s,co,a), v] = sum_{k in win(s)} Wt[k][s*out_blk + (co,a)] X[k, v] + bias[(s,co,a)]
 // (= sum_k W[(s,co,a)][k] X[k, v]).  When tc_forward_reads_w(d) (no per-shell column
@@ -60,12 +69,13 @@ bool tc_gemm_supported(const LscDims& d, int64_t n_vox, int64_t ld_in, int64_t l
 bool tc_forward_reads_w(const LscDims& d);
 cudaError_t tc_lsc_forward(const LscDims& d, const void* X, const void* W, const void* Wt, const float* bias, void* Y,
                            int64_t n_vox, int64_t ldx, int64_t ldy, int* err_word, cudaStream_t st,
-                           TcParts parts = TcParts{});
+                           TcParts parts = TcParts{}, TcLeaky act = TcLeaky{});
 // dX[(s',ci,b), v] = sum_{k in rwin(s')} W[k][s'*in_blk + (ci,b)] dY[k, v].  Reads Wt (K-major)
 // when tc_dgrad_reads_wt and Wt is given, else W.
 bool tc_dgrad_reads_wt(const LscDims& d, int64_t n_vox, bool split);
 cudaError_t tc_lsc_dgrad(const LscDims& d, const void* dY, const void* W, const void* Wt, void* dX, int64_t n_vox,
-                         int64_t lddy, int64_t lddx, int* err_word, cudaStream_t st, TcParts parts = TcParts{});
+                         int64_t lddy, int64_t lddx, int* err_word, cudaStream_t st, TcParts parts = TcParts{},
+                         TcLeaky act = TcLeaky{});
 // P[split][(s,co,a)][(s',ci,b)] = sum_{v in split} dY[(s,co,a), v] X[(s',ci,b), v] for s' in win(s),
 // P[split][(s,co,a)][rows_in] = sum_{v in split} dY[(s,co,a), v] (BF16; with split operands
 // split_bf16x3_sums writes them).  The partials are stored transposed, P[split][col][row] with leading dimension ldp >= rows_out (the row

@@ -126,9 +126,11 @@ def lsc_workspace(geom: L.LSCGeometry, n_vox: int, c_in: int, c_out: int, dtype,
 
 
 def lsc_forward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, b: torch.Tensor | None, c_in: int,
-                c_out: int, out: torch.Tensor | None = None, workspace=None) -> torch.Tensor:
+                c_out: int, out: torch.Tensor | None = None, workspace=None,
+                slope: float | None = None) -> torch.Tensor:
     """``workspace``: optional (tensor, ptr, bytes) from lsc_workspace; a backward-sized
-    workspace lets the following backward reuse the operator built here."""
+    workspace lets the following backward reuse the operator built here.  ``slope``: a leaky
+    ReLU on the output, in the same call."""
     x = as_act(x)
     n_vox = x.shape[1]
     if out is None:
@@ -138,9 +140,13 @@ def lsc_forward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, b: torch.
     w = w.detach().contiguous().float()
     bf = b.detach().contiguous().float() if b is not None else None  # lives until after the launch
     bp = bf.data_ptr() if bf is not None else None
-    L.check(L.get().delimit_lsc_forward(geom.handle, x.data_ptr(), w.data_ptr(), bp, out.data_ptr(), n_vox, c_in,
-                                        c_out, x.stride(0), out.stride(0), _code(x), 0, wsp, ws_n, _stream()),
-            "delimit_lsc_forward")
+    args = (n_vox, c_in, c_out, x.stride(0), out.stride(0), _code(x), 0, wsp, ws_n, _stream())
+    if slope is None:
+        L.check(L.get().delimit_lsc_forward(geom.handle, x.data_ptr(), w.data_ptr(), bp, out.data_ptr(), *args),
+                "delimit_lsc_forward")
+    else:
+        L.check(L.get().delimit_lsc_forward_leaky(geom.handle, x.data_ptr(), w.data_ptr(), bp, out.data_ptr(),
+                                                  float(slope), *args), "delimit_lsc_forward_leaky")
     return out
 
 
@@ -171,8 +177,9 @@ def lsc_forward_sh2signal(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor,
 
 def lsc_backward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, d_out: torch.Tensor, c_in: int, c_out: int,
                  need_input: bool = True, need_weight: bool = True, need_bias: bool = True, workspace=None,
-                 operator_ready: bool = False):
-    """``workspace`` + ``operator_ready``: reuse the operator a forward built in this workspace."""
+                 operator_ready: bool = False, slope: float | None = None):
+    """``workspace`` + ``operator_ready``: reuse the operator a forward built in this workspace.
+    ``slope``: x is a leaky ReLU's output and d_in the gradient of that leaky ReLU's input."""
     x = as_act(x)
     d_out = as_act(d_out.to(x.dtype))
     n_vox = x.shape[1]
@@ -189,17 +196,28 @@ def lsc_backward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, d_out: t
     if workspace is None:
         workspace, operator_ready = lsc_workspace(geom, n_vox, c_in, c_out, x.dtype, True, x.device), False
     _, wsp, ws_n = workspace
-    L.check(L.get().delimit_lsc_backward(
-        geom.handle, x.data_ptr(), w.data_ptr(), d_out.data_ptr(), d_in.data_ptr() if d_in is not None else None,
-        dw.data_ptr() if dw is not None else None, db.data_ptr() if db is not None else None, n_vox, c_in, c_out,
-        x.stride(0), d_out.stride(0), _code(x), L.OPERATOR_READY if operator_ready else 0, wsp, ws_n, _stream()),
-        "delimit_lsc_backward")
+    ptrs = (geom.handle, x.data_ptr(), w.data_ptr(), d_out.data_ptr(), d_in.data_ptr() if d_in is not None else None,
+            dw.data_ptr() if dw is not None else None, db.data_ptr() if db is not None else None)
+    args = (n_vox, c_in, c_out, x.stride(0), d_out.stride(0), _code(x), L.OPERATOR_READY if operator_ready else 0, wsp,
+            ws_n, _stream())
+    if slope is None:
+        L.check(L.get().delimit_lsc_backward(*ptrs, *args), "delimit_lsc_backward")
+    else:
+        L.check(L.get().delimit_lsc_backward_leaky(*ptrs, float(slope), *args), "delimit_lsc_backward_leaky")
     return d_in, dw, db
 
 
 # ---------------------------------------------------------------------------
 # autograd
 # ---------------------------------------------------------------------------
+def _untracked(*tensors) -> bool:
+    """Nothing follows these tensors: no gradient recorded, no forward-mode level, no tracer and no
+    function transform, so that a Function's bookkeeping (about 10 us a call) can be left out."""
+    return (not (torch.is_grad_enabled() and any(t is not None and t.requires_grad for t in tensors))
+            and torch.autograd.forward_ad._current_level < 0 and torch._C._get_tracing_state() is None
+            and torch._C._functorch.peek_interpreter_stack() is None)
+
+
 class _TransformFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, basis, kind, channels, out_dtype):
@@ -234,6 +252,72 @@ class _LSCFn(torch.autograd.Function):
                                     operator_ready=ctx.ws is not None)
         ctx.ws = None
         return d_in, dw, db, None, None, None
+
+
+class _LSCStackFn(torch.autograd.Function):
+    """LSC layers with a leaky ReLU between them, activations and gradients as the single layers
+    make them, the leaky ReLU and its adjoint in the GEMMs' epilogues (a pass over the
+    activations less per layer and direction)."""
+
+    @staticmethod
+    def forward(ctx, x, slope, layers, *params):  # layers: (geom, c_in, c_out); params: w, b of each in turn
+        ctx.slope, ctx.layers = slope, layers
+        ctx.has_b = [b is not None for b in params[1::2]]
+        hs, ctx.ws = [x], []
+        for i, (geom, c_in, c_out) in enumerate(layers):
+            # a backward-sized workspace: the backward reuses the operator built here
+            ctx.ws.append(lsc_workspace(geom, x.shape[1], c_in, c_out, x.dtype, True, x.device))
+            hs.append(lsc_forward(geom, hs[-1], params[2 * i], params[2 * i + 1], c_in, c_out, workspace=ctx.ws[i],
+                                  slope=slope if i + 1 < len(layers) else None))
+        ctx.save_for_backward(*hs[:-1], *params[::2])
+        return hs[-1]
+
+    @staticmethod
+    def backward(ctx, g):
+        n = len(ctx.layers)
+        hs, ws = ctx.saved_tensors[:n], ctx.saved_tensors[n:]
+        grads = [None] * (2 * n)
+        for i in reversed(range(n)):
+            geom, c_in, c_out = ctx.layers[i]
+            need_x = i > 0 or ctx.needs_input_grad[0]
+            g, grads[2 * i], grads[2 * i + 1] = lsc_backward(
+                geom, hs[i], ws[i], g, c_in, c_out, need_input=need_x, need_weight=ctx.needs_input_grad[3 + 2 * i],
+                need_bias=ctx.has_b[i] and ctx.needs_input_grad[4 + 2 * i], workspace=ctx.ws[i],
+                operator_ready=ctx.ws[i] is not None, slope=ctx.slope if i > 0 else None)
+            ctx.ws[i] = None
+        return (g, None, None, *grads)
+
+
+def _plain(m: torch.nn.Module, cls) -> bool:
+    """m is exactly a cls and nothing watches or replaces its calls."""
+    return type(m) is cls and "forward" not in m.__dict__ and not (
+        m._forward_hooks or m._forward_pre_hooks or m._backward_hooks or m._backward_pre_hooks
+        or getattr(m, "_compiled_call_impl", None))
+
+
+def lsc_stack(x: torch.Tensor, lscs, act) -> torch.Tensor:
+    """lscs[-1](act(... act(lscs[0](x)))).  LSC layers and a LeakyReLU of this module on 2-D
+    activations run with the leaky ReLU inside the layers' kernels; anything else (other modules,
+    subclasses, hooks on a module) is called as it is."""
+    g = torch.nn.modules.module
+    lscs = list(lscs)
+    if not (x.dim() == 2 and len(lscs) > 1 and _plain(act, LeakyReLU)
+            and all(_plain(m, LocalSphericalConvolution) for m in lscs)
+            and not (g._global_forward_hooks or g._global_forward_pre_hooks or g._global_backward_hooks
+                     or g._global_backward_pre_hooks)):
+        for i, m in enumerate(lscs):
+            x = m(x if i == 0 else act(x))
+        return x
+    params = [(m.point_weights(), m.bias) for m in lscs]
+    i = 0  # layers that no gradient flows through keep nothing for a backward
+    while i < len(lscs) and _untracked(x, *params[i]):
+        m = lscs[i]
+        x = lsc_forward(m.geom, x, *params[i], m.c_in, m.c_out, slope=act.slope if i + 1 < len(lscs) else None)
+        i += 1
+    if i == len(lscs):
+        return x
+    return _LSCStackFn.apply(x, act.slope, [(m.geom, m.c_in, m.c_out) for m in lscs[i:]],
+                             *(p for wb in params[i:] for p in wb))
 
 
 def leaky_relu(x: torch.Tensor, slope: float) -> torch.Tensor:

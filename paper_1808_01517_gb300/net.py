@@ -97,11 +97,7 @@ class SphericalNet(torch.nn.Module):
     def forward_sh(self, h: torch.Tensor) -> torch.Tensor:
         """From the input's SH coefficients (the Signal2SH output, e.g. of a gathered,
         b0-normalised load) to the [270, V] prediction."""
-        for i, lsc in enumerate(self.lscs):
-            h = lsc(h)
-            if i < len(self.lscs) - 1:
-                h = self.act(h)
-        return self.sh2s(h)
+        return self.sh2s(layers.lsc_stack(h, self.lscs, self.act))
 
 
 class Fallback:
