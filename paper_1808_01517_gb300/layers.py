@@ -25,8 +25,16 @@ def _code(t: torch.Tensor) -> int:
     return _DT[t.dtype]
 
 
+# The current stream's handle without building a Stream object (0.4 us a call against 3), where
+# this torch has the call.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_cur_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _cur_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_cur_device())
 
 
 def padded_ld(n_vox: int) -> int:
@@ -36,7 +44,14 @@ def padded_ld(n_vox: int) -> int:
 
 def empty_act(rows: int, n_vox: int, dtype, device="cuda") -> torch.Tensor:
     """[rows, n_vox] view of a [rows, padded_ld] buffer (the library's activation layout)."""
-    return torch.empty((rows, padded_ld(n_vox)), dtype=dtype, device=device)[:, :n_vox]
+    ld = padded_ld(n_vox)
+    buf = torch.empty((rows, ld), dtype=dtype, device=device)
+    return buf if ld == n_vox else buf[:, :n_vox]  # (a slice costs as much as a launch)
+
+
+def _f32(w: torch.Tensor) -> torch.Tensor:
+    """w as contiguous float32 (itself when it is)."""
+    return w if w.dtype is torch.float32 and w.is_contiguous() else w.detach().contiguous().float()
 
 
 def _is_act(x: torch.Tensor) -> bool:
@@ -137,8 +152,8 @@ def lsc_forward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, b: torch.
         out = empty_act(geom.s_out * c_out * geom.n_out, n_vox, x.dtype, x.device)
     _, wsp, ws_n = workspace if workspace is not None else lsc_workspace(geom, n_vox, c_in, c_out, x.dtype, False,
                                                                          x.device)
-    w = w.detach().contiguous().float()
-    bf = b.detach().contiguous().float() if b is not None else None  # lives until after the launch
+    w = _f32(w)
+    bf = _f32(b) if b is not None else None  # lives until after the launch
     bp = bf.data_ptr() if bf is not None else None
     args = (n_vox, c_in, c_out, x.stride(0), out.stride(0), _code(x), 0, wsp, ws_n, _stream())
     if slope is None:
@@ -166,8 +181,8 @@ def lsc_forward_sh2signal(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor,
         out = empty_act(c_out * geom.out_basis.n_dirs, n_vox, x.dtype, x.device)
     _, wsp, ws_n = workspace if workspace is not None else lsc_workspace(geom, n_vox, c_in, c_out, x.dtype, False,
                                                                          x.device)
-    w = w.detach().contiguous().float()
-    bf = b.detach().contiguous().float() if b is not None else None  # lives until after the launch
+    w = _f32(w)
+    bf = _f32(b) if b is not None else None  # lives until after the launch
     L.check(L.get().delimit_lsc_forward_sh2signal(geom.handle, x.data_ptr(), w.data_ptr(),
                                                   bf.data_ptr() if bf is not None else None, out.data_ptr(), n_vox,
                                                   c_in, c_out, x.stride(0), out.stride(0), _code(x), 0, wsp, ws_n,
@@ -190,8 +205,8 @@ def lsc_backward(geom: L.LSCGeometry, x: torch.Tensor, w: torch.Tensor, d_out: t
         d_in = torch.empty((x.shape[0], x.stride(0)), dtype=x.dtype, device=x.device)
         if x.stride(0) != n_vox:
             d_in = d_in[:, :n_vox]
-    w = w.detach().contiguous().float()
-    dw = torch.empty_like(w) if need_weight else None
+    w = _f32(w)
+    dw = torch.empty(w.shape, dtype=torch.float32, device=w.device) if need_weight else None
     db = torch.empty((c_out, geom.s_out), dtype=torch.float32, device=x.device) if need_bias else None
     if workspace is None:
         workspace, operator_ready = lsc_workspace(geom, n_vox, c_in, c_out, x.dtype, True, x.device), False
@@ -385,6 +400,8 @@ class Signal2SH(torch.nn.Module):
 
     def forward(self, signal):
         x, restore = _to_rows(signal)
+        if _untracked(x):
+            return restore(transform("signal2sh", self.basis, x, self.channels, self.out_dtype))
         return restore(_TransformFn.apply(x, self.basis, "signal2sh", self.channels, self.out_dtype))
 
 
@@ -400,6 +417,8 @@ class SH2Signal(torch.nn.Module):
 
     def forward(self, sh):
         x, restore = _to_rows(sh)
+        if _untracked(x):
+            return restore(transform("sh2signal", self.basis, x, self.channels, self.out_dtype))
         return restore(_TransformFn.apply(x, self.basis, "sh2signal", self.channels, self.out_dtype))
 
 
@@ -475,4 +494,7 @@ class LocalSphericalConvolution(torch.nn.Module):
 
     def forward(self, sh):
         x, restore = _to_rows(sh)
-        return restore(_LSCFn.apply(x, self.point_weights(), self.bias, self.geom, self.c_in, self.c_out))
+        w = self.point_weights()
+        if _untracked(x, w, self.bias):  # a forward-sized workspace will do
+            return restore(lsc_forward(self.geom, x, w, self.bias, self.c_in, self.c_out))
+        return restore(_LSCFn.apply(x, w, self.bias, self.geom, self.c_in, self.c_out))
