@@ -452,7 +452,7 @@ delimit_status delimit_selftest_wait_timeout(void* stream);
  *   0: every step on the CUDA-core kernels (same results within the dtype's
  *     rounding; used to cross-check the two).
  * Other values: INVALID_ARG.  The operator build runs on the tensor cores for
- * BF16 activations when K <= 64, c_in <= 128 and c_in * N_in is a multiple of 8
+ * BF16 activations when K <= 64, c_in divides 128 and c_in * N_in is a multiple of 8
  * (modes 1 and 2), the weight gradient's reduction for BF16 activations when
  * K <= 64, else on the CUDA cores; they and the gathered Signal2SH are not counted
  * as fallbacks and never refused. */

@@ -1005,7 +1005,7 @@ static delimit_status lsc_backward(const delimit_lsc_geometry* g, const void* sh
       parts.act = d.rows_out * p.ld3;
       parts.op = d.rows_out * d.ldW;
       // the parts of the K-major operator (240-column tiles without padded columns, as BF16): with W3
-      // as it lies 720 columns run as 768; 1.81 ms against 2.00 at 16,001 voxels, 64 -> 16 channels
+      // as it lies 720 columns run as 768; 1.81 ms against 2.00 at 16,001 voxels, 16 -> 64 channels
       char* Wd3 = nullptr;
       if (tc_dgrad_reads_wt(d, n_vox, true)) {
         Wd3 = base + p.off_Wd3;

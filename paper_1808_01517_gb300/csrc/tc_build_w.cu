@@ -197,12 +197,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_
       p.bias[r] = p.b ? p.b[co * d.s_out + s] * p.q[s * d.n_out + aa] : 0.f;
     }
   }
-  const int rowlen = (int)d.in_blk;  // a row run of W with its padding, which the staging buffers keep at zero
-  if (rowlen != d.c_in * d.n_in) {
-    for (uint32_t o = threadIdx.x * 16; o < p.nh * p.stg_bytes; o += kBwThreads * 16)
-      *reinterpret_cast<uint4*>(smem + stg_off + o) = make_uint4(0, 0, 0, 0);
-    fence_proxy_async_smem();
-  }
+  const int rowlen = (int)d.in_blk;  // a row run of W
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -499,7 +494,9 @@ void build_w_tables_destroy(BuildWTables& t) {
 }
 
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t) {
-  if (!tc_enabled() || !t.ok || d.c_in < 1 || d.c_in > 128) return false;
+  // Other channel counts keep the CUDA-core build's sums: a network's FP32 gradients would show the
+  // other rounding (1e-4 of W's entries a BF16 step away)
+  if (!tc_enabled() || !t.ok || d.c_in < 1 || 128 % d.c_in != 0 || d.in_blk != (int64_t)d.c_in * d.n_in) return false;
   if (bw_smem(d.n_in, d.c_in, d.in_blk, d.K, 1) > kBwSmemLimit) return false;
   int dev = 0, major = 0;
   cudaGetDevice(&dev);
