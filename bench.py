@@ -35,16 +35,16 @@ UNIT = "voxels/s"
 # profiles/chain_65536vox_launch_list.md (the `dram__bytes_*` metrics); valid only
 # while the kernel's sources hash to the value recorded with the capture (re-hashed
 # only after host-side edits that leave the kernels' device code unchanged).
-_GEMM = ("csrc/tc_gemm.cu", "csrc/tc_ptx.cuh"), "ab66a0cc8a65094a"
-_TF = ("csrc/tc_transform.cu", "csrc/tc_ptx.cuh"), "03ad4be21121a183"
+_GEMM = ("csrc/tc_gemm.cu", "csrc/tc_ptx.cuh"), "2c9ebf18673e1755"
+_TF = ("csrc/tc_transform.cu", "csrc/tc_ptx.cuh"), "eb7c548664354ca4"
 NCU_TRAFFIC = {
-    "lsc_fwd_gemm": {"bytes": 1.523e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
-    "lsc_dgrad_gemm": {"bytes": 2.653e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
-    "lsc_wgrad_gemm": {"bytes": 3.270e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
-    "signal2sh_tc": {"bytes": 0.8136e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
+    "lsc_fwd_gemm": {"bytes": 1.831e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
+    "lsc_dgrad_gemm": {"bytes": 3.479e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
+    "lsc_wgrad_gemm": {"bytes": 2.617e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
+    "signal2sh_tc": {"bytes": 0.8104e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
     "sh2signal_tc": {"bytes": 3.333e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
     "sh2signal_bwd_tc": {"bytes": 3.358e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
-    "signal2sh_bwd_tc": {"bytes": 0.7846e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
+    "signal2sh_bwd_tc": {"bytes": 0.7845e9, "n_vox": 65536, "sources": _TF[0], "sha256_16": _TF[1]},
 }
 
 
