@@ -328,7 +328,9 @@ __global__ void __launch_bounds__(f32_threads(TMA), 1) transform_tc_f32_kernel(c
       fetch();
     }
     for (int i = 0; i < n_chunks; ++i) {
-      if (kGroups > 1 && (i & 1) != grp) {  // the other group's chunk
+      // The other group's chunk.  Its stage's lap may go by unwatched: chunks are consumed in order, and
+      // this group's chunk before waited for one that comes after that lap (two stages or more).
+      if (kGroups > 1 && (i & 1) != grp) {
         ss.next();
         continue;
       }
