@@ -1122,8 +1122,8 @@ static delimit_status lsc_backward(const delimit_lsc_geometry* g, const void* sh
       if (e != cudaSuccess) return cuda_fail(e, "LSC weight-gradient launch");
     }
     float* dwp = reinterpret_cast<float*>(base + p.off_dwp);
-    // BF16 activations: the reduction on the tensor cores (its error, that of an FP32 sum, is far
-    // below the voxel sums'); FP32 ones keep FP32 FMAs
+    // BF16 activations: the reduction on the tensor cores, at the error of the FP32 sum (measured in
+    // tc_reduce_dw.cu); FP32 ones keep FP32 FMAs
     if (act_t == DELIMIT_BF16 && tc && tc_reduce_dw_supported(g->rd))
       e = tc_reduce_dw(d, g->rd, P, p_cs, split_stride, p.splits, g->d_q, dw, db, dwp, g->err_word, cs);
     else

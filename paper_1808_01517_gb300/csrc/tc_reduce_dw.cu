@@ -3,15 +3,21 @@
 // per shell pair a GEMM [channel pairs] x [(b,a) entries] x [kernel points k < K <= 64],
 // from the FP32 partials P that the weight-gradient GEMM stored transposed (a column
 // (s',ci,b) holds its rows (s,co,a) contiguously).  FP32 operands as three-part BF16
-// splits, six part products, FP32 accumulation over at most one part of the b range
-// (about 250 (b,a) entries, the sums of the parts added in FP32): the error of the FP32 sum
-// it replaces, which is far below that of the voxel sums in G itself.
+// splits, six part products.  A tensor-core accumulator cuts every addition off toward zero, so
+// the products x0 M0, which carry the sum, meet few others there: two k-steps of 16 coefficients,
+// the second added to the first, then the accumulator is read and added up in FP32 registers.  The
+// products 2^-8 and 2^-16 of them have accumulators of their own, read once per part of the b range.
+// Relative error of dw against FP64 (64 -> 64 channels): 16 voxels 1.1e-7 against 1.7e-7 for the FP32
+// sum on the CUDA cores, 300 voxels 3.2e-7 against 3.2e-7, 8,192 voxels (the voxel sums') 4.4e-6
+// against 4.4e-6; all products of a part in one accumulator gave 1.9e-6, 2.1e-6 and 6.0e-6.
 //
-// What bounds it: reading P (58 MB per split at 16 -> 64 channels, 232 MB at 64 -> 64).  On
-// the CUDA cores the step was bound by issue instead (64 FMAs per (b,a) entry and pair).
-// Measured, with the sum of the parts and db: 64 -> 64 channels, 2 splits 0.123 ms (4.5 TB/s of
-// P in the main kernel) against 0.353 on the CUDA cores; 16 -> 64 channels, 3 splits 0.053
-// against 0.106.
+// What bounds it: the thread that issues the MMAs, about 100 cycles each at these widths and 450 for
+// a group's wait and commit, then reading P (58 MB per split at 16 -> 64 channels, 232 MB at
+// 64 -> 64).  M's parts side by side in N make four MMAs of the six products of a k-step; six of them
+// with the same groups took 0.096 ms in the main kernel where this takes 0.092 (64 -> 64, one split).
+// On the CUDA cores the step was bound by issue (64 FMAs per (b,a) entry and pair).  Measured, with
+// the sum of the parts and db: 64 -> 64 channels, one split 0.111 ms against 0.342 on the CUDA
+// cores, four splits 0.122 against 0.346; 16 -> 64 channels 0.038 and 0.050 against 0.095 and 0.100.
 //
 // A persistent CTA walks units (shell s, part of the b range, input shell s', tile of up to
 // 128 channel pairs), consecutive units sharing the part's M images in shared memory:
@@ -21,8 +27,9 @@
 //     floats: an odd stride, no bank conflicts for odd n_out), split the sum into BF16 parts and
 //     store them to TMEM as the MMA's A operand (no shared-memory round trip);
 //   - one thread issues the MMAs (A from TMEM, M images MN-major from shared memory);
-//   - four warps read the accumulator and store the partial sums, lanes along the pairs.
+//   - eight warps read the accumulators, add them up and store the partial sums, lanes along the pairs.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "tc_gemm.h"
@@ -34,12 +41,17 @@ namespace {
 
 constexpr int kRdN = 64;          // kernel points (MMA N), zero-padded
 constexpr int kRdConvWarps = 16;  // four per TMEM lane quarter
-constexpr int kRdThreads = 32 * (2 + 4 + kRdConvWarps);
+constexpr int kRdEpiWarps = 8;    // two per TMEM lane quarter, 32 kernel points each
+constexpr int kRdConv0 = 2 + kRdEpiWarps;  // first converter warp
+constexpr int kRdThreads = 32 * (kRdConv0 + kRdConvWarps);
 constexpr int kRdMaxKs = 8;       // k-steps of 16 output coefficients per b
 constexpr int kRdRing = 6;        // most ring slots
-constexpr int kRdABufs = 4;       // most A buffers
+constexpr uint32_t kRdACols = 24; // a k-step of A: three parts of 16 coefficients, two to a column
 constexpr size_t kRdSmemLimit = 226 * 1024;
-constexpr uint32_t kRdDCols = 2 * kRdN;
+// TMEM: an accumulator of x0 M0 for every other group of two k-steps; one of x0 M1 + x1 M0 and one of
+// x0 M2 + x1 M1 + x2 M0 for every other unit; the A buffers of two groups
+constexpr uint32_t kRdSmall = 2 * kRdN, kRdA = kRdSmall + 4 * kRdN, kRdABuf = 2 * kRdACols;
+static_assert(kRdA + 2 * kRdABuf <= 512, "TMEM columns");
 
 enum : int {
   kErrRdRing = 0x5100,
@@ -47,7 +59,6 @@ enum : int {
   kErrRdA = 0x5300,
   kErrRdAEmpty = 0x5400,
   kErrRdD = 0x5500,
-  kErrRdDEmpty = 0x5600,
   kErrRdB = 0x5700,
   kErrRdDrain = 0x5800
 };
@@ -91,7 +102,7 @@ struct RdParams {
   int64_t ldpt, split_stride, part_stride, rows_total;
   int splits, ks, bpp, nparts;
   int nseg, co_chunks, ntiles;  // a tile: nseg input channels x all c_out, or one channel x 128 outputs
-  int ring, abufs;
+  int ring;
   uint32_t seg_stride, ring_bytes, img_bytes;  // img_bytes: one b's image
   int64_t units;
   int pg_per_pair;
@@ -134,6 +145,8 @@ struct RdUnit {
   }
 };
 
+// PER_B: most k-steps of an input coefficient that one warp converts
+template <int PER_B>
 __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __grid_constant__ RdParams p) {
   using namespace ptx;
   extern __shared__ uint8_t smem_raw[];
@@ -142,18 +155,15 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
   const uint32_t sbase = smem_u32(smem);
   const uint32_t ring_off = (uint32_t)p.bpp * p.img_bytes;  // [images of a part][ring slots][barriers]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ring_off + (uint32_t)p.ring * p.ring_bytes);
-  // bars: ring_full[6], ring_empty[6], a_full[4], a_empty[4], d_full[2], d_empty[2], b_full, b_empty, drain
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kRdRing + 2 * kRdABufs + 7);
+  // bars: ring_full[6], ring_empty[6], full[2], done[2], b_full, b_empty, drain
+  uint64_t* bars2 = bars + 2 * kRdRing;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars2 + 7);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   auto ring_full = [&](int i) { return smem_u32(bars + i); };
   auto ring_empty = [&](int i) { return smem_u32(bars + kRdRing + i); };
-  auto a_full = [&](int i) { return smem_u32(bars + 2 * kRdRing + i); };
-  auto a_empty = [&](int i) { return smem_u32(bars + 2 * kRdRing + kRdABufs + i); };
-  auto d_full = [&](int i) { return smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + i); };
-  auto d_empty = [&](int i) { return smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 2 + i); };
-  const uint32_t b_full = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 4);
-  const uint32_t b_empty = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 5);
-  const uint32_t drain_bar = smem_u32(bars + 2 * kRdRing + 2 * kRdABufs + 6);
+  auto full = [&](int i) { return smem_u32(bars2 + i); };      // a group's A is there, its accumulators are free
+  auto done = [&](int i) { return smem_u32(bars2 + 2 + i); };  // a group's MMAs: its A is free, its sums are there
+  const uint32_t b_full = smem_u32(bars2 + 4), b_empty = smem_u32(bars2 + 5), drain_bar = smem_u32(bars2 + 6);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 
   if (threadIdx.x == 0) {
@@ -161,13 +171,9 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
       mbar_init(ring_full(i), 1);
       mbar_init(ring_empty(i), kRdConvWarps);
     }
-    for (int i = 0; i < kRdABufs; ++i) {
-      mbar_init(a_full(i), kRdConvWarps);
-      mbar_init(a_empty(i), 1);
-    }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(d_full(i), 1);
-      mbar_init(d_empty(i), 4);
+      mbar_init(full(i), kRdConvWarps / 2 + kRdEpiWarps);
+      mbar_init(done(i), 1);
     }
     mbar_init(b_full, 1);
     mbar_init(b_empty, 1);
@@ -183,7 +189,6 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const uint32_t a_cols = (uint32_t)(24 * p.ks);  // TMEM columns of one A buffer: 3 parts x 8 per k-step
   // this CTA's consecutive units
   const int64_t u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
   const int cw = d.c_out < 128 ? d.c_out : 128;  // output channels of a full tile row of segments
@@ -248,95 +253,133 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
     if (lane == 0) {
       RdUnit un;
       un.init(p, u0);
-      const uint32_t idesc = idesc_bf16(128, kRdN, false, true);
+      const uint32_t idesc1 = idesc_bf16(128, kRdN, false, true), idesc2 = idesc_bf16(128, 2 * kRdN, false, true);
       const uint32_t part_bytes = (uint32_t)p.ks * 2048u;
-      int key = -1, buf = 0;
-      uint32_t a_ph = 0, b_ph = 0;
+      const uint64_t part = part_bytes >> 4, img = p.img_bytes >> 4;
+      const uint64_t bd0 = umma_desc(sbase, part_bytes, 1024, kSwizzle128B);
+      int key = -1;
+      uint32_t grp = 0, b_ph = 0;  // groups so far
       bool ok = true;
       for (int64_t u = u0; u < u1 && ok && !*abort_flag; ++u) {
-        const int acc = (int)((u - u0) & 1);
-        const uint32_t d_use = (uint32_t)(((u - u0) >> 1) & 1);
-        const int nb = min(p.bpp, d.n_in - un.part * p.bpp);
+        const int steps = min(p.bpp, d.n_in - un.part * p.bpp) * p.ks;
         if (un.key(p) != key) {
           key = un.key(p);
           if (!wait_bounded(b_full, b_ph, abort_flag, p.err, kErrRdB)) break;
           b_ph ^= 1u;
         }
-        if (!wait_bounded(d_empty(acc), d_use ^ 1u, abort_flag, p.err, kErrRdDEmpty)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kRdN);
-        for (int b = 0; b < nb; ++b) {
-          if (!wait_bounded(a_full(buf), a_ph, abort_flag, p.err, kErrRdA)) {
-            ok = false;
-            break;
-          }
+        const uint32_t small = tmem_base + kRdSmall + (uint32_t)((u - u0) & 1) * (2 * kRdN);
+        uint64_t bd = bd0;  // the k-step's image, by additions (a descriptor built per MMA took longer than the MMA)
+        int kk = 0;
+        for (int t = 0; t < steps; t += 2, ++grp) {
+          const uint32_t set = grp & 1, lead = tmem_base + set * kRdN, x = tmem_base + kRdA + set * kRdABuf;
+          if (!(ok = wait_bounded(full(set), (grp >> 1) & 1u, abort_flag, p.err, kErrRdA))) break;
           tc_fence_after();
-          const uint32_t a_tmem = tmem_base + kRdDCols + (uint32_t)buf * a_cols;
-          // operand addresses by one addition each: a descriptor built per MMA took longer than the MMA
-          const uint64_t bd0 = umma_desc(sbase + (uint32_t)b * p.img_bytes, part_bytes, 1024, kSwizzle128B);
-          for (int kk = 0; kk < p.ks; ++kk) {
-#pragma unroll
-            for (int pr = 0; pr < 6; ++pr) {  // part products, smallest first
-              constexpr int pa[6] = {2, 1, 0, 1, 0, 0}, pb[6] = {0, 1, 2, 0, 1, 0};
-              mma_bf16_ts(d_tmem, a_tmem + (uint32_t)(pa[pr] * 8 * p.ks + kk * 8), bd0 + pb[pr] * (part_bytes >> 4) + kk * 128,
-                          idesc, (b | kk | pr) != 0);
+          // four MMAs for the six part products of a k-step
+          auto step = [&](uint32_t xi, uint32_t acc_lead, uint32_t acc_small) {
+            mma_bf16_ts(lead, xi, bd, idesc1, acc_lead);                               // x0 M0
+            mma_bf16_ts(small, xi, bd + part, idesc2, acc_small);                      // x0 [M1 M2]
+            mma_bf16_ts(small, xi + kRdACols / 3, bd, idesc2, 1);                      // x1 [M0 M1]
+            mma_bf16_ts(small + kRdN, xi + 2 * kRdACols / 3, bd, idesc1, 1);           // x2 M0
+            bd += 128;
+            if (++kk == p.ks) {  // the next input coefficient's image
+              kk = 0;
+              bd += img - part;
             }
-          }
-          mma_commit(a_empty(buf));
-          if (++buf == p.abufs) {
-            buf = 0;
-            a_ph ^= 1u;
-          }
+          };
+          step(x, 0, t > 0);
+          if (t + 1 < steps) step(x + kRdACols, 1, 1);
+          mma_commit(done(set));
         }
         if (!ok) break;
-        mma_commit(d_full(acc));
         un.next(p);
         if (u + 1 < u1 && un.key(p) != key) mma_commit(b_empty);
       }
       mma_commit(drain_bar);
       wait_drain(drain_bar, 0, p.err, kErrRdDrain);
     }
-  } else if (warp < 6) {
-    // ---- epilogue: lane = channel pair of the tile, columns = kernel points ----
-    const int q = warp & 3, r = q * 32 + lane;
+  } else if (warp < kRdConv0) {
+    // ---- epilogue: lane = channel pair of the tile, columns = kernel points, 32 per warp of a quarter;
+    // the groups' accumulators, then the small products', added up in FP32 registers ----
+    const int q = warp & 3, h0 = 32 * ((warp - 2) >> 2), r = q * 32 + lane;
+    const uint32_t tl = tmem_base + ((uint32_t)(q * 32) << 16) + h0;
+    if (lane == 0) {  // both accumulators are free
+      mbar_arrive(full(0));
+      mbar_arrive(full(1));
+    }
+    uint32_t grp = 0;
+    bool ok = true;
     RdUnit un;
     un.init(p, u0);
-    for (int64_t u = u0; u < u1; ++u, un.next(p)) {
-      const int acc = (int)((u - u0) & 1);
-      const bool ok = wait_bounded_sleep(d_full(acc), (uint32_t)(((u - u0) >> 1) & 1), abort_flag, p.err, kErrRdD);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      tc_fence_after();
-      const uint32_t tl = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kRdN);
+    for (int64_t u = u0; u < u1 && ok; ++u, un.next(p)) {
+      const int steps = min(p.bpp, d.n_in - un.part * p.bpp) * p.ks;
+      float sum[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) sum[k] = 0.f;
+      for (int t = 0; t < steps; t += 2, ++grp) {
+        const uint32_t set = grp & 1;
+        ok = wait_bounded_sleep(done(set), (grp >> 1) & 1u, abort_flag, p.err, kErrRdD);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        tc_fence_after();
+        if (h0 < d.K) {
+          uint32_t x[16];
+#pragma unroll
+          for (int h = 0; h < 32; h += 16) {
+            tmem_ld16_nowait(tl + set * kRdN + h, x);
+            tmem_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[h + k] += __uint_as_float(x[k]);
+          }
+          if (t + 2 >= steps) {  // the unit's last group: read before its accumulator is given back, so that a
+                                 // unit's first group finds the small products of the unit before last read
+            const uint32_t small = kRdSmall + (uint32_t)((u - u0) & 1) * (2 * kRdN);
+#pragma unroll
+            for (int h = 0; h < 32; h += 8) {
+              uint32_t y[8], z[8];
+              tmem_ld8_nowait(tl + small + kRdN + h, y);
+              tmem_ld8_nowait(tl + small + h, z);
+              tmem_wait_ld();
+#pragma unroll
+              for (int k = 0; k < 8; ++k) sum[h + k] += __uint_as_float(y[k]) + __uint_as_float(z[k]);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full(set));
+      }
+      if (!ok) break;
       const int co0 = d.c_out < 128 ? 0 : (un.tile % p.co_chunks) * 128;
       const int ci0 = d.c_out < 128 ? un.tile * p.nseg : un.tile / p.co_chunks;
       const int g = r / cw, co = co0 + r - g * cw;
-      const bool valid = g < p.nseg && ci0 + g < d.c_in && co < d.c_out;
-      float* out = p.dwp + un.part * p.part_stride +
-                   (((int64_t)un.s * d.s_in + un.sp) * d.c_in + ci0 + g) * d.c_out + co;
+      if (g < p.nseg && ci0 + g < d.c_in && co < d.c_out) {
+        float* out = p.dwp + un.part * p.part_stride + h0 * p.rows_total +
+                     (((int64_t)un.s * d.s_in + un.sp) * d.c_in + ci0 + g) * d.c_out + co;
 #pragma unroll
-      for (int h = 0; h < kRdN; h += 32) {
-        uint32_t rv[2][16];
-        tmem_ld16_nowait(tl + h, rv[0]);
-        tmem_ld16_nowait(tl + h + 16, rv[1]);
-        tmem_wait_ld();
-        if (valid) {
-#pragma unroll
-          for (int k = 0; k < 32; ++k)
-            if (h + k < d.K) out[(h + k) * p.rows_total] = __uint_as_float(rv[k >> 4][k & 15]);
-        }
+        for (int k = 0; k < 32; ++k)
+          if (h0 + k < d.K) out[k * p.rows_total] = sum[k];
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(d_empty(acc));
     }
   } else {
-    // ---- converters: lane = channel pair; warp `sub` of a quarter takes every fourth k-step ----
-    const int q = warp & 3, sub = (warp - 6) >> 2, r = q * 32 + lane;
+    // ---- converters: lane = channel pair; of the four warps of a quarter two take every other group, a
+    // k-step each ----
+    const int q = warp & 3, sub = (warp - kRdConv0) >> 2, r = q * 32 + lane;
     const int g = r / cw, cl = r - g * cw;
+    const uint32_t set = (uint32_t)sub >> 1, at = tmem_base + ((uint32_t)(q * 32) << 16) + kRdA + set * kRdABuf + (sub & 1) * kRdACols;
+    uint32_t fills = 0;  // groups this warp has converted
+    auto wait_done = [&]() {  // the group before it in this set is done
+      const bool w = wait_bounded_sleep(done(set), (fills & 1u) ^ 1u, abort_flag, p.err, kErrRdAEmpty);
+      return (bool)__all_sync(0xffffffffu, w);
+    };
+    auto give = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full(set));
+      ++fills;
+    };
     RdUnit un;
     un.init(p, u0);
-    int slot = 0, buf = 0;
-    uint32_t ph = 0, a_ph = 0;
+    int slot = 0;
+    uint32_t ph = 0, grp = 0;  // grp: the unit's first group
     bool ok = true;
     for (int64_t u = u0; u < u1 && ok; ++u, un.next(p)) {
       const int nb = min(p.bpp, d.n_in - un.part * p.bpp);
@@ -345,13 +388,15 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
       const bool valid = g < p.nseg && ci0 + g < d.c_in && co0 + cl < d.c_out;
       const int mis = (int)((((int64_t)un.s * d.c_out + co0) * d.n_out) & 3);
       const uint32_t lane_off = valid ? (uint32_t)g * p.seg_stride + (uint32_t)(mis + cl * d.n_out) * 4u : 0u;
+      // this warp's k-steps of the unit: place sub & 1 of every group with the parity of `set`
+      const int first = (sub & 1) + 2 * (int)((set ^ grp) & 1u);
       for (int b = 0; b < nb && ok; ++b) {
-        const int kk0 = (sub - b * p.ks) & 3;  // this warp's k-steps of this b: kk0, kk0 + 4
-        float v[kRdMaxKs / 4][16];
+        const int kk0 = (first - b * p.ks) & 3;  // of this b: kk0, kk0 + 4
+        float v[PER_B][16];
 #pragma unroll
-        for (int i = 0; i < kRdMaxKs / 4; ++i)
+        for (int j = 0; j < PER_B; ++j)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[i][j] = 0.f;
+          for (int e = 0; e < 16; ++e) v[j][e] = 0.f;
         for (int z = 0; z < p.splits; ++z) {
           ok = wait_bounded_sleep(ring_full(slot), ph, abort_flag, p.err, kErrRdRing);
           ok = __all_sync(0xffffffffu, ok);
@@ -359,15 +404,15 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
           if (valid) {
             const float* src = reinterpret_cast<const float*>(smem + ring_off + (uint32_t)slot * p.ring_bytes + lane_off);
 #pragma unroll
-            for (int i = 0; i < kRdMaxKs / 4; ++i) {
-              const int a0 = 16 * (kk0 + 4 * i);
+            for (int j = 0; j < PER_B; ++j) {
+              const int a0 = 16 * (kk0 + 4 * j);
               if (a0 + 16 <= d.n_out) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[i][j] += src[a0 + j];
+                for (int e = 0; e < 16; ++e) v[j][e] += src[a0 + e];
               } else if (a0 < d.n_out) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  if (a0 + j < d.n_out) v[i][j] += src[a0 + j];
+                for (int e = 0; e < 16; ++e)
+                  if (a0 + e < d.n_out) v[j][e] += src[a0 + e];
               }
             }
           }
@@ -379,36 +424,31 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
           }
         }
         if (!ok) break;
-        ok = wait_bounded_sleep(a_empty(buf), a_ph ^ 1u, abort_flag, p.err, kErrRdAEmpty);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + kRdDCols + (uint32_t)buf * a_cols;
 #pragma unroll
-        for (int i = 0; i < kRdMaxKs / 4; ++i) {
-          const int kk = kk0 + 4 * i;
-          if (kk < p.ks) {
-            uint32_t part[3][8];
+        for (int j = 0; j < PER_B; ++j) {
+          if (kk0 + 4 * j >= p.ks) break;
+          if (!(ok = wait_done())) break;
+          tc_fence_after();
+          uint32_t part[3][8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              uint32_t t3[3];
-              split3x2(v[i][2 * j], v[i][2 * j + 1], t3);
+          for (int e = 0; e < 8; ++e) {
+            uint32_t t3[3];
+            split3x2(v[j][2 * e], v[j][2 * e + 1], t3);
 #pragma unroll
-              for (int t = 0; t < 3; ++t) part[t][j] = t3[t];
-            }
-#pragma unroll
-            for (int t = 0; t < 3; ++t) tmem_st8(at + (uint32_t)(t * 8 * p.ks + kk * 8), part[t]);
+            for (int t = 0; t < 3; ++t) part[t][e] = t3[t];
           }
-        }
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(a_full(buf));
-        if (++buf == p.abufs) {
-          buf = 0;
-          a_ph ^= 1u;
+#pragma unroll
+          for (int t = 0; t < 3; ++t) tmem_st8(at + (uint32_t)(t * 8), part[t]);
+          tmem_wait_st();
+          give();
         }
       }
+      // an odd number of k-steps: the last group has one, and its other warp has nothing to convert
+      const int steps = nb * p.ks, groups = (steps + 1) / 2;
+      if (ok && (steps & 1) && (sub & 1) && ((grp + groups - 1) & 1u) == set) {
+        if ((ok = wait_done())) give();
+      }
+      grp += groups;
     }
   }
   tc_fence_before();
@@ -493,7 +533,7 @@ int rd_bpp(int n_in, int n_out) {
 // shared memory beside the ring: the part's images, alignment and barriers
 size_t rd_fixed(int n_in, int n_out) {
   const int ks = (n_out + 15) / 16;
-  return 1024 + (size_t)rd_bpp(n_in, n_out) * 3 * ks * 2048 + (2 * kRdRing + 2 * kRdABufs + 7) * 8 + 64;
+  return 1024 + (size_t)rd_bpp(n_in, n_out) * 3 * ks * 2048 + (2 * kRdRing + 7) * 8 + 64;
 }
 
 }  // namespace
@@ -562,21 +602,21 @@ cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float*
   p.pg_per_pair = d.m_stride_sp ? 1 : 0;
   p.err = err;
   for (int s = 0; s < d.s_out; ++s) p.units += (int64_t)p.nparts * std::max(0, d.win_hi[s] - d.win_lo[s]) * p.ntiles;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaError_t e;
   if (dw && p.units > 0) {
     const size_t fixed = rd_fixed(d.n_in, d.n_out);
     p.ring = (int)std::min<size_t>(kRdRing, (kRdSmemLimit - fixed) / p.ring_bytes);
     if (p.ring < 2) return cudaErrorInvalidValue;
-    p.abufs = std::min(kRdABufs, (int)((512 - kRdDCols) / (24 * p.ks)));
     // at least 120 KiB so that two CTAs never share an SM (each holds 512 TMEM columns)
     const size_t smem = std::max<size_t>(120 * 1024, fixed + (size_t)p.ring * p.ring_bytes);
-    e = cudaFuncSetAttribute(reduce_dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = p.ks > 4 ? reduce_dw_tc_kernel<2> : reduce_dw_tc_kernel<1>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned grid = (unsigned)std::min<int64_t>(p.units, std::max(1, sms));
-    reduce_dw_tc_kernel<<<grid, kRdThreads, smem, st>>>(p);
+    kern<<<grid, kRdThreads, smem, st>>>(p);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
