@@ -482,8 +482,8 @@ uint64_t delimit_cuda_core_fallbacks(void);
  * (lsc_build_w_tc on the tensor cores), lsc_fwd_gemm, lsc_dgrad_gemm,
  * lsc_wgrad_gemm (the _f32 suffix for split FP32 operands), lsc_fwd_sh2signal (the
  * fused LSC forward + SH2Signal), lsc_rowsum (single-CTA BF16 path),
- * lsc_transpose_w, split_bf16x3, lsc_reduce_dw, signal2sh_gather, lsc_gemm_simt,
- * lsc_wgrad_simt.
+ * lsc_transpose_w, split_bf16x3, lsc_reduce_dw (lsc_reduce_dw_tc on the tensor cores),
+ * signal2sh_gather, lsc_gemm_simt, lsc_wgrad_simt.
  * No counterpart in the paper. */
 delimit_status delimit_trace_enable(int enable);
 int64_t delimit_trace_summary(char* buf, size_t cap);

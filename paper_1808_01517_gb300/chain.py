@@ -188,6 +188,7 @@ class Chain:
             "lsc_build_w": (build, wbytes),
             "lsc_build_w_tc": (build, wbytes),
             "lsc_reduce_dw": (build, 4.0 * r["c_out"] * r["c_in"]),
+            "lsc_reduce_dw_tc": (build, 4.0 * r["c_out"] * r["c_in"]),
             "lsc_rowsum": (1.0 * r["c_out"] * V, e * V * r["c_out"]),
             "signal2sh_tc": (fl["signal2sh"], by["signal2sh"]),
             "sh2signal_tc": (fl["sh2signal"], by["sh2signal"]),

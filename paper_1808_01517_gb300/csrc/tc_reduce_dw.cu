@@ -578,7 +578,7 @@ bool tc_reduce_dw_supported(const ReduceDwTables& t) {
 
 cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float* P, int64_t ldpt, int64_t split_stride,
                          int splits, const float* q, float* dw, float* db, float* scratch, int* err, cudaStream_t st) {
-  TraceScope trace("lsc_reduce_dw", st);
+  TraceScope trace("lsc_reduce_dw_tc", st);
   RdParams p;
   memset(&p, 0, sizeof p);
   p.d = d;
