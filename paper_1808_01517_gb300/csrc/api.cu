@@ -1124,7 +1124,7 @@ static delimit_status lsc_backward(const delimit_lsc_geometry* g, const void* sh
     float* dwp = reinterpret_cast<float*>(base + p.off_dwp);
     // BF16 activations: the reduction on the tensor cores, at the error of the FP32 sum (measured in
     // tc_reduce_dw.cu); FP32 ones keep FP32 FMAs
-    if (act_t == DELIMIT_BF16 && tc && tc_reduce_dw_supported(g->rd))
+    if (act_t == DELIMIT_BF16 && tc && tc_reduce_dw_supported(d, g->rd))
       e = tc_reduce_dw(d, g->rd, P, p_cs, split_stride, p.splits, g->d_q, dw, db, dwp, g->err_word, cs);
     else
       e = launch_reduce_dw(d, P, p_rs, p_cs, split_stride, p.splits, g->d_M, g->d_Mt, g->d_q, dw, db, dwp, cs);

@@ -127,7 +127,7 @@ struct ReduceDwTables {
 cudaError_t reduce_dw_tables_create(const LscDims& dims_template, const float* d_M, ReduceDwTables& t,
                                     std::string& err);
 void reduce_dw_tables_destroy(ReduceDwTables& t);
-bool tc_reduce_dw_supported(const ReduceDwTables& t);
+bool tc_reduce_dw_supported(const LscDims& d, const ReduceDwTables& t);
 // dw and db as launch_reduce_dw from the transposed partials; scratch: reduce_dw_scratch_floats(d)
 cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float* P, int64_t ldpt, int64_t split_stride,
                          int splits, const float* q, float* dw, float* db, float* scratch, int* err, cudaStream_t st);

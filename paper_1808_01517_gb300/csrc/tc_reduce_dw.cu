@@ -16,8 +16,8 @@
 // 64 -> 64).  M's parts side by side in N make four MMAs of the six products of a k-step; six of them
 // with the same groups took 0.096 ms in the main kernel where this takes 0.092 (64 -> 64, one split).
 // On the CUDA cores the step was bound by issue (64 FMAs per (b,a) entry and pair).  Measured, with
-// the sum of the parts and db: 64 -> 64 channels, one split 0.111 ms against 0.342 on the CUDA
-// cores, four splits 0.122 against 0.346; 16 -> 64 channels 0.038 and 0.050 against 0.095 and 0.100.
+// the sum of the parts and db: 64 -> 64 channels, one split 0.110 ms against 0.342 on the CUDA
+// cores, four splits 0.121 against 0.346; 16 -> 64 channels 0.035 and 0.047 against 0.095 and 0.100.
 //
 // A persistent CTA walks units (shell s, part of the b range, input shell s', tile of up to
 // 128 channel pairs), consecutive units sharing the part's M images in shared memory:
@@ -462,26 +462,27 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
 // dw = sum of the parts in order (zero outside the window), 32 pairs x K points per block through
 // shared memory ([k][pair] in, [pair][k] out), and db in the blocks after them, one warp per
 // (co, s): db[co,s] = sum_a q[s][a] (row sum of dY's row (s,co,a) over the splits)
-__global__ void __launch_bounds__(256) finish_dw_kernel(const __grid_constant__ RdParams p, float* __restrict__ dw,
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) finish_dw_kernel(const __grid_constant__ RdParams p, float* __restrict__ dw,
                                                         float* __restrict__ db, const float* __restrict__ qv,
                                                         int64_t dw_blocks) {
   __shared__ float t[kRdN][33];
   const LscDims& d = p.d;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   if ((int64_t)blockIdx.x < dw_blocks) {
-    const int64_t r0 = (int64_t)blockIdx.x * 32, row = r0 + lane;
-    auto decode = [&](int64_t r, int& s, int& sp, int& ci, int& co) {
-      co = (int)(r % d.c_out);
+    const uint32_t r0 = blockIdx.x * 32, row = r0 + lane;  // rows_total < 2^31 (tc_reduce_dw_supported)
+    auto decode = [&](uint32_t r, uint32_t& s, uint32_t& sp, uint32_t& ci, uint32_t& co) {
+      co = r % d.c_out;
       r /= d.c_out;
-      ci = (int)(r % d.c_in);
+      ci = r % d.c_in;
       r /= d.c_in;
-      sp = (int)(r % d.s_in);
-      s = (int)(r / d.s_in);
+      sp = r % d.s_in;
+      s = r / d.s_in;
     };
-    int s, sp, ci, co;
+    uint32_t s, sp, ci, co;
     decode(row < p.rows_total ? row : 0, s, sp, ci, co);
-    const bool in = row < p.rows_total && sp >= d.win_lo[s] && sp < d.win_hi[s];
-    for (int k = warp; k < d.K; k += 8) {
+    const bool in = row < p.rows_total && (int)sp >= d.win_lo[s] && (int)sp < d.win_hi[s];
+    for (int k = warp; k < d.K; k += WARPS) {
       float a = 0.f;
       if (in) {  // eight parts' loads in flight, summed in order
         const float* src = p.dwp + k * p.rows_total + row;
@@ -496,14 +497,14 @@ __global__ void __launch_bounds__(256) finish_dw_kernel(const __grid_constant__ 
       t[k][lane] = a;
     }
     __syncthreads();
-    for (int i = warp; i < 32; i += 8) {
+    for (int i = warp; i < 32; i += WARPS) {
       if (r0 + i >= p.rows_total) break;
       decode(r0 + i, s, sp, ci, co);
       float* out = dw + ((((int64_t)co * d.s_out + s) * d.c_in + ci) * d.s_in + sp) * d.K;
       for (int k = lane; k < d.K; k += 32) out[k] = t[k][i];
     }
   } else {
-    const int64_t i = ((int64_t)blockIdx.x - dw_blocks) * 8 + warp;
+    const int64_t i = ((int64_t)blockIdx.x - dw_blocks) * WARPS + warp;
     if (i >= (int64_t)d.c_out * d.s_out) return;
     const int co = (int)(i / d.s_out), s = (int)(i % d.s_out);
     const int64_t row0 = ((int64_t)s * d.c_out + co) * d.n_out;
@@ -568,8 +569,13 @@ void reduce_dw_tables_destroy(ReduceDwTables& t) {
   t = ReduceDwTables();
 }
 
-bool tc_reduce_dw_supported(const ReduceDwTables& t) {
-  if (!t.ok || !tc_enabled()) return false;
+bool tc_reduce_dw_supported(const LscDims& d, const ReduceDwTables& t) {
+  if (!t.ok || !tc_enabled() || (int64_t)d.s_out * d.s_in * d.c_in * d.c_out > INT32_MAX) return false;
+  // A tile copies a run of P per input channel, and more than 32 short ones a step take longer than
+  // the CUDA cores' loads.  us, here and there, 64 -> 1 channels 26 / 24 at 2,048 voxels and 64 / 58 at
+  // 16,384 (64 runs of 180 bytes), 64 -> 2 27 / 24 and 65 / 59; 64 -> 4 20 / 34 and 42 / 67 (32 runs),
+  // 16 -> 1 17 / 23 and 27 / 24.
+  if (std::min(128 / std::min(d.c_out, 128), d.c_in) > 32) return false;
   int dev = 0, major = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
@@ -622,10 +628,19 @@ cudaError_t tc_reduce_dw(const LscDims& d, const ReduceDwTables& t, const float*
     if (e != cudaSuccess) return e;
   }
   const int64_t dw_blocks = dw ? (p.rows_total + 31) / 32 : 0;
-  const int64_t db_blocks = db ? ((int64_t)d.c_out * d.s_out + 7) / 8 : 0;
-  if (dw_blocks + db_blocks == 0) return cudaSuccess;
-  finish_dw_kernel<<<(unsigned)(dw_blocks + db_blocks), 256, 0, st>>>(p, dw, db, q, dw_blocks);
-  count_launch();
+  // 32 warps a block (a warp per kernel point or two, so that the parts' loads are all in flight) where
+  // two such blocks per SM hold them all, else eight.  us with 32 and with eight: 1 -> 64 channels
+  // 4.0 / 6.0, 16 -> 64 6.4 / 9.5, 16 -> 16 of order 10 (18 parts) 6.2 / 11.5, 64 -> 64 20.9 / 18.0
+  auto finish = [&](auto kern, int warps) {
+    const int64_t db_blocks = db ? ((int64_t)d.c_out * d.s_out + warps - 1) / warps : 0;
+    if (dw_blocks + db_blocks == 0) return;
+    kern<<<(unsigned)(dw_blocks + db_blocks), 32 * warps, 0, st>>>(p, dw, db, q, dw_blocks);
+    count_launch();
+  };
+  if (dw_blocks <= 2 * sms)
+    finish(finish_dw_kernel<32>, 32);
+  else
+    finish(finish_dw_kernel<8>, 8);
   return cudaGetLastError();
 }
 

@@ -22,6 +22,11 @@ CASES = {
     "resampling_free": ([40, 40, 40], 8, 8, 3, 2, 6, "adjacent", True, 8, 12, "bf16", True),
     # 120 output coefficients: eight k-steps of one input coefficient
     "order14": ([128], 4, 14, 1, 2, 6, "same", False, 4, 20, "bf16", True),
+    "64_to_4": ([40, 40], 8, 8, 2, 2, 6, "adjacent", False, 64, 4, "bf16", True),
+    "16_to_1": ([40, 40], 8, 8, 2, 2, 6, "adjacent", False, 16, 1, "bf16", True),
+    # more than 32 short runs a step
+    "64_to_1": ([40, 40], 8, 8, 2, 2, 6, "adjacent", False, 64, 1, "bf16", False),
+    "33_to_3": ([40, 40], 8, 8, 2, 2, 6, "adjacent", False, 33, 3, "bf16", False),
     # more than 64 kernel points
     "k73": ([40, 40], 8, 8, 2, 6, 12, "adjacent", False, 3, 5, "bf16", False),
     # the M images of 45 input coefficients in one part: more than a CTA's shared memory
