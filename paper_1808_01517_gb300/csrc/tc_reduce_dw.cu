@@ -109,6 +109,22 @@ struct RdParams {
   int* err;
 };
 
+// split3x2 for any FP32 value: the first two parts keep within the largest BF16 value, so that what a
+// sum has beyond it, infinity or NaN included, is left to the last part.  That one meets M0 alone: the
+// products have the sign (or the NaN) that the FP32 product has, and no infinity meets M1 and M2,
+// whose signs differ from M's.  One instruction per pair and part: 92.7 us against 92.3 in the main kernel
+// at 64 -> 64 channels (with fminf and fmaxf 97).
+__device__ __forceinline__ void split3x2_any(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    // at most the largest BF16 value in magnitude (for NaN, the largest value)
+    asm("min.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(p[q]) : "r"(ptx::pack_bf16x2f(x, y)), "r"(0x7F7F7F7Fu));
+    x -= __uint_as_float(p[q] << 16);
+    y -= __uint_as_float(p[q] & 0xFFFF0000u);
+  }
+  p[2] = ptx::pack_bf16x2f(x, y);
+}
+
 // one unit of work and its walk: (s, part, s', tile), tile fastest
 struct RdUnit {
   int s, part, sp, tile;
@@ -427,16 +443,16 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
 #pragma unroll
         for (int j = 0; j < PER_B; ++j) {
           if (kk0 + 4 * j >= p.ks) break;
-          if (!(ok = wait_done())) break;
-          tc_fence_after();
           uint32_t part[3][8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             uint32_t t3[3];
-            split3x2(v[j][2 * e], v[j][2 * e + 1], t3);
+            split3x2_any(v[j][2 * e], v[j][2 * e + 1], t3);
 #pragma unroll
             for (int t = 0; t < 3; ++t) part[t][e] = t3[t];
           }
+          if (!(ok = wait_done())) break;
+          tc_fence_after();
 #pragma unroll
           for (int t = 0; t < 3; ++t) tmem_st8(at + (uint32_t)(t * 8), part[t]);
           tmem_wait_st();
