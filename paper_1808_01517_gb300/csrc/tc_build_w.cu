@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_
     un.init(p, u0);
     int key = -1, slot = 0, m_loads = 0;
     uint32_t ph = 0;
-    for (int64_t u = u0; u < u1 && !*abort_flag; ++u, un.next(p)) {
+    for (int64_t u = u0; u < u1 && !warp_aborted(abort_flag); ++u, un.next(p)) {
       bool ok = wait_bounded(w_empty(slot), ph ^ 1u, abort_flag, p.err, kErrBwWEmpty);
       if (!__all_sync(0xffffffffu, ok)) break;
       if (warp == 0 && un.key(p) != key) {

@@ -72,6 +72,10 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, vola
   }
 }
 
+// Whether *abort is raised, the same answer for every lane (a whole warp's loop condition: a lane that
+// left alone would be waited for at the next warp barrier, without a limit).
+__device__ __forceinline__ bool warp_aborted(volatile int* abort) { return __any_sync(0xffffffffu, *abort != 0); }
+
 // try_wait with a suspend-time hint: the thread sleeps until the phase completes or
 // about `hint_ns` pass, instead of returning at once (fewer issue slots while waiting).
 __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity, uint32_t hint_ns) {

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kRdThreads, 1) reduce_dw_tc_kernel(const __gri
     uint32_t used = 0;  // ring slots that have been filled
     int b_loads = 0;
     bool ok = true;
-    for (int64_t u = u0; u < u1 && ok && !*abort_flag; ++u, un.next(p)) {
+    for (int64_t u = u0; u < u1 && ok && !warp_aborted(abort_flag); ++u, un.next(p)) {
       const int b0 = un.part * p.bpp, nb = min(p.bpp, d.n_in - b0);
       if (un.key(p) != key) {
         // the images of the units before are read by MMAs that have completed
