@@ -660,7 +660,7 @@ cudaError_t launch_build_w(const LscDims& d, const float* w, const float* b, con
   const int nab = d.n_out * d.n_in, npairs = d.c_out * d.c_in;
   cudaError_t e;
   const int64_t blocks = (int64_t)((npairs + kBwP - 1) / kBwP) * d.s_out * d.s_in * ((nab + kBwAB - 1) / kBwAB);
-  if (!Wt && blocks < 152) {  // fewer blocks than SMs
+  if (!Wt && blocks < sm_count()) {
     const dim3 grid((unsigned)((npairs + kBwsPairs - 1) / kBwsPairs), (unsigned)(d.s_out * d.s_in),
                     (unsigned)((nab + kBwsThreads - 1) / kBwsThreads));
     if (w_t == 0)
