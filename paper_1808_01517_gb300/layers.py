@@ -247,16 +247,21 @@ class _TransformFn(torch.autograd.Function):
 
 
 class _LSCFn(torch.autograd.Function):
+    """``slope_out``: a leaky ReLU on the output; the gradient that arrives is the one of that leaky
+    ReLU's input.  ``slope_in``: x is such an output; the gradient handed on is the one of that leaky
+    ReLU's input.  Both in the GEMMs' epilogues (a pass over the activations less per layer and
+    direction); lsc_stack sets them in pairs on neighbouring layers."""
+
     @staticmethod
-    def forward(ctx, x, w, b, geom, c_in, c_out):
-        ctx.geom, ctx.c_in, ctx.c_out = geom, c_in, c_out
+    def forward(ctx, x, w, b, geom, c_in, c_out, slope_out=None, slope_in=None):
+        ctx.geom, ctx.c_in, ctx.c_out, ctx.slope_in = geom, c_in, c_out, slope_in
         ctx.has_b = b is not None
         ctx.save_for_backward(x, w)
         # a backward-sized workspace: the backward reuses the operator built here
         ws = lsc_workspace(geom, x.shape[1], c_in, c_out, x.dtype, True, x.device) \
             if any(ctx.needs_input_grad) else None
         ctx.ws = ws
-        return lsc_forward(geom, x, w, b, c_in, c_out, workspace=ws)
+        return lsc_forward(geom, x, w, b, c_in, c_out, workspace=ws, slope=slope_out)
 
     @staticmethod
     def backward(ctx, g):
@@ -264,43 +269,9 @@ class _LSCFn(torch.autograd.Function):
         d_in, dw, db = lsc_backward(ctx.geom, x, w, g, ctx.c_in, ctx.c_out, need_input=ctx.needs_input_grad[0],
                                     need_weight=ctx.needs_input_grad[1],
                                     need_bias=ctx.has_b and ctx.needs_input_grad[2], workspace=ctx.ws,
-                                    operator_ready=ctx.ws is not None)
+                                    operator_ready=ctx.ws is not None, slope=ctx.slope_in)
         ctx.ws = None
-        return d_in, dw, db, None, None, None
-
-
-class _LSCStackFn(torch.autograd.Function):
-    """LSC layers with a leaky ReLU between them, activations and gradients as the single layers
-    make them, the leaky ReLU and its adjoint in the GEMMs' epilogues (a pass over the
-    activations less per layer and direction)."""
-
-    @staticmethod
-    def forward(ctx, x, slope, layers, *params):  # layers: (geom, c_in, c_out); params: w, b of each in turn
-        ctx.slope, ctx.layers = slope, layers
-        ctx.has_b = [b is not None for b in params[1::2]]
-        hs, ctx.ws = [x], []
-        for i, (geom, c_in, c_out) in enumerate(layers):
-            # a backward-sized workspace: the backward reuses the operator built here
-            ctx.ws.append(lsc_workspace(geom, x.shape[1], c_in, c_out, x.dtype, True, x.device))
-            hs.append(lsc_forward(geom, hs[-1], params[2 * i], params[2 * i + 1], c_in, c_out, workspace=ctx.ws[i],
-                                  slope=slope if i + 1 < len(layers) else None))
-        ctx.save_for_backward(*hs[:-1], *params[::2])
-        return hs[-1]
-
-    @staticmethod
-    def backward(ctx, g):
-        n = len(ctx.layers)
-        hs, ws = ctx.saved_tensors[:n], ctx.saved_tensors[n:]
-        grads = [None] * (2 * n)
-        for i in reversed(range(n)):
-            geom, c_in, c_out = ctx.layers[i]
-            need_x = i > 0 or ctx.needs_input_grad[0]
-            g, grads[2 * i], grads[2 * i + 1] = lsc_backward(
-                geom, hs[i], ws[i], g, c_in, c_out, need_input=need_x, need_weight=ctx.needs_input_grad[3 + 2 * i],
-                need_bias=ctx.has_b[i] and ctx.needs_input_grad[4 + 2 * i], workspace=ctx.ws[i],
-                operator_ready=ctx.ws[i] is not None, slope=ctx.slope if i > 0 else None)
-            ctx.ws[i] = None
-        return (g, None, None, *grads)
+        return d_in, dw, db, None, None, None, None, None
 
 
 def _plain(m: torch.nn.Module, cls) -> bool:
@@ -323,16 +294,17 @@ def lsc_stack(x: torch.Tensor, lscs, act) -> torch.Tensor:
         for i, m in enumerate(lscs):
             x = m(x if i == 0 else act(x))
         return x
-    params = [(m.point_weights(), m.bias) for m in lscs]
-    i = 0  # layers that no gradient flows through keep nothing for a backward
-    while i < len(lscs) and _untracked(x, *params[i]):
-        m = lscs[i]
-        x = lsc_forward(m.geom, x, *params[i], m.c_in, m.c_out, slope=act.slope if i + 1 < len(lscs) else None)
-        i += 1
-    if i == len(lscs):
-        return x
-    return _LSCStackFn.apply(x, act.slope, [(m.geom, m.c_in, m.c_out) for m in lscs[i:]],
-                             *(p for wb in params[i:] for p in wb))
+    # a node per layer: a layer's gradients arrive, and what it kept is freed, before the next one's
+    # backward, as with the modules
+    slope_in = None
+    for i, m in enumerate(lscs):
+        w, b, slope = m.point_weights(), m.bias, act.slope if i + 1 < len(lscs) else None
+        if _untracked(x, w, b):  # no gradient flows through it: nothing is kept for a backward
+            x = lsc_forward(m.geom, x, w, b, m.c_in, m.c_out, slope=slope)
+        else:
+            x = _LSCFn.apply(x, w, b, m.geom, m.c_in, m.c_out, slope, slope_in)
+        slope_in = slope
+    return x
 
 
 def leaky_relu(x: torch.Tensor, slope: float) -> torch.Tensor:
