@@ -351,7 +351,11 @@ delimit_status delimit_lsc_forward_sh2signal_supported(const delimit_lsc_geometr
  *   geometry, sizes, dtype and w built in this workspace (b is not needed here).
  * All outputs are overwritten (not accumulated).  Reductions over voxels are
  * deterministic (fixed split and order).
- *   workspace >= delimit_lsc_workspace_size(..., 1) bytes, 256-byte aligned.
+ *   workspace >= delimit_lsc_workspace_size(..., 1) bytes, 256-byte aligned.  For F32 from
+ *   4,096 voxels on, c_in N_in a multiple of 240 and c_out N_out of 8, its last
+ *   6 S_in c_in N_in S_out c_out N_out bytes (rounded up to 256) hold the operator
+ *   transposed for the input gradient; a buffer without them is taken too, and the input
+ *   gradient then reads the operator as it lies (about a tenth slower).
  * n_vox = 0 writes zeros to dw and db.  w is needed only for d_in, sh_in only for
  * dw or db.  Errors as delimit_lsc_forward, with d_out, sh_in and d_in checked
  * like its activations. */

@@ -804,7 +804,8 @@ static delimit_status lsc_common_checks(const delimit_lsc_geometry* g, int64_t n
     return fail(DELIMIT_ERR_INVALID_ARG, "need n_vox >= 0, 1 <= c_in, c_out <= 4096 and a valid dtype");
   delimit_status st = check_device(g->device);
   if (st != DELIMIT_OK) return st;
-  const size_t need = bwd ? p.total_bwd : p.total_fwd;
+  // the input gradient's transposed parts, at the end, are left out where the buffer ends before them
+  const size_t need = bwd ? p.off_Wd3 : p.total_fwd;
   if (ws_bytes < need) {
     char buf[128];
     std::snprintf(buf, sizeof buf, "workspace %zu bytes < %zu needed", ws_bytes, need);
@@ -1007,7 +1008,7 @@ static delimit_status lsc_backward(const delimit_lsc_geometry* g, const void* sh
       // the parts of the K-major operator (240-column tiles without padded columns, as BF16): with W3
       // as it lies 720 columns run as 768; 1.81 ms against 2.00 at 16,001 voxels, 16 -> 64 channels
       char* Wd3 = nullptr;
-      if (tc_dgrad_reads_wt(d, n_vox, true)) {
+      if (tc_dgrad_reads_wt(d, n_vox, true) && ws_bytes >= p.total_bwd) {
         Wd3 = base + p.off_Wd3;
         for (int q = 0; q < 3; ++q) {
           e = transpose_bf16(base + p.off_W3 + size_t(q) * d.rows_out * d.ldW * 2, d.rows_out, d.ldW, d.ldW,
