@@ -384,7 +384,8 @@ delimit_status delimit_lsc_backward_leaky(const delimit_lsc_geometry* geom, cons
  * between LSC layers, applied to SH coefficients).  x and y may alias. */
 delimit_status delimit_leaky_relu(const void* x, void* y, int64_t rows, int64_t n_vox, int64_t ld_x, int64_t ld_y,
                                   float slope, delimit_dtype dtype, void* stream);
-/* dx = dy * (y > 0 ? 1 : slope), with y the forward output (it keeps the input's sign). */
+/* dx = dy * (y > 0 ? 1 : slope), with y the forward output (it keeps the input's sign).  dy and
+ * dx may alias (the same pointer and row stride). */
 delimit_status delimit_leaky_relu_backward(const void* y, const void* dy, void* dx, int64_t rows, int64_t n_vox,
                                            int64_t ld_y, int64_t ld_dy, int64_t ld_dx, float slope,
                                            delimit_dtype dtype, void* stream);

@@ -49,9 +49,9 @@ __global__ void leaky_bf16x8_kernel(const __nv_bfloat16* x, __nv_bfloat16* y, in
   }
 }
 
-__global__ void leaky_bwd_bf16x8_kernel(const __nv_bfloat16* __restrict__ y, const __nv_bfloat16* __restrict__ dy,
-                                        __nv_bfloat16* __restrict__ dx, int64_t n, int64_t ldy, int64_t lddy,
-                                        int64_t lddx, float slope) {
+// (dx may be dy: neither is __restrict__)
+__global__ void leaky_bwd_bf16x8_kernel(const __nv_bfloat16* __restrict__ y, const __nv_bfloat16* dy, __nv_bfloat16* dx,
+                                        int64_t n, int64_t ldy, int64_t lddy, int64_t lddx, float slope) {
   const int64_t r = blockIdx.y;
   const int64_t n8 = n / 8;
   const uint4* yr = reinterpret_cast<const uint4*>(y + r * ldy);
@@ -84,8 +84,8 @@ static bool al16(const void* p, int64_t ld) {
 
 // dx = dy * (y > 0 ? 1 : slope): the forward output y carries the sign of its input
 template <typename T>
-__global__ void leaky_bwd_kernel(const T* __restrict__ y, const T* __restrict__ dy, T* __restrict__ dx, int64_t rows,
-                                 int64_t n, int64_t ldy, int64_t lddy, int64_t lddx, float slope) {
+__global__ void leaky_bwd_kernel(const T* __restrict__ y, const T* dy, T* dx, int64_t rows, int64_t n, int64_t ldy,
+                                 int64_t lddy, int64_t lddx, float slope) {
   const int64_t r = blockIdx.y;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const float a = ld1(y + r * ldy + v), g = ld1(dy + r * lddy + v);

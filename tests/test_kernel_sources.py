@@ -38,3 +38,15 @@ def test_a_warp_leaves_its_loop_together():
             single = any("lane == 0" in h for h in _enclosing_headers(text, m.start()))
             assert single, (os.path.basename(path), text[:m.start()].count("\n") + 1)
     assert reads >= 10
+
+
+def test_in_place_kernels_do_not_declare_their_buffers_apart():
+    """delimit_leaky_relu and its backward run in place (dx = dy, as the layers' backward calls it):
+    __restrict__ on those two would promise the compiler the opposite."""
+    text = _source("elementwise.cu")
+    for kernel, names in (("leaky_kernel", "xy"), ("leaky_bf16x8_kernel", "xy"),
+                          ("leaky_bwd_kernel", ("dy", "dx")), ("leaky_bwd_bf16x8_kernel", ("dy", "dx"))):
+        params = re.search(r"void " + kernel + r"\(([^)]*)\)", text).group(1)
+        for name in names:
+            assert re.search(r"\* " + name + r"\b", params), (kernel, name, params)
+            assert not re.search(r"__restrict__ " + name + r"\b", params), (kernel, name, params)
