@@ -8,7 +8,6 @@
 //   reduce_dw        dW -> kernel-point weights dw and bias gradient db
 #include <algorithm>
 #include <atomic>
-#include <type_traits>
 
 #include "kernels.h"
 
@@ -126,18 +125,13 @@ __device__ __forceinline__ void st_y4(__nv_bfloat16* p, float a, float b, float 
   *reinterpret_cast<uint2*>(p) = u;
 }
 
-// GATHER: output voxel v reads input column a.index[v] scaled by 1 / a.b0[index[v]]
-// (plain loads into an FP32 tile: columns are not contiguous).
-template <typename Tin, typename Tout, bool GATHER>
+template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(32 * (kTfMaxOut / kTfOpt)) transform_staged_kernel(const __grid_constant__ TransformArgs a,
                                                                                      int n_groups, int og_count,
                                                                                      int max_in) {
-  using Ts = typename std::conditional<GATHER, float, Tin>::type;  // type of the staged input tile
   extern __shared__ float4 tf_smem4[];
   float* Tt = reinterpret_cast<float*>(tf_smem4);                 // [max_in][12 * og_count]
-  Ts* Xs = reinterpret_cast<Ts*>(Tt + max_in * kTfOpt * og_count);  // [max_in][128]
-  int64_t* sidx = reinterpret_cast<int64_t*>(Xs + max_in * kTfVox);  // GATHER: source column per voxel
-  float* sinv = reinterpret_cast<float*>(sidx + kTfVox);            // GATHER: 1 / b0 per voxel
+  Tin* Xs = reinterpret_cast<Tin*>(Tt + max_in * kTfOpt * og_count);  // [max_in][128]
   const int ldt = kTfOpt * og_count;
   const int tid = threadIdx.x, q = tid % 32, og = tid / 32;
   const int64_t vt_count = (a.n_vox + kTfVox - 1) / kTfVox;
@@ -153,46 +147,16 @@ __global__ void __launch_bounds__(32 * (kTfMaxOut / kTfOpt)) transform_staged_ke
     const int64_t v0 = (r % vt_count) * kTfVox;
     const TransformGroup& G = a.g[g];
     __syncthreads();  // the previous tile's reads of Xs (and Tt) are done
-    if (GATHER) {
-      // source columns and b0 factors of this tile's voxels, then every input row
-      for (int vv = tid; vv < kTfVox; vv += blockDim.x) {  // the block may have fewer than 128 threads
-        const int64_t v = v0 + vv;
-        int64_t src = -1;
-        float inv = 0.f;
-        if (v < a.n_vox) {
-          src = a.index[v];
-          if (src < 0 || src >= a.n_src) {
-            if (a.err) atomicCAS(a.err, 0, kErrGatherIndex);
-            src = -1;
-          } else if (a.b0) {
-            const float b = a.b0[src];
-            inv = b > 0.f ? 1.f / b : 0.f;
-          } else {
-            inv = 1.f;
-          }
-        }
-        sidx[vv] = src;
-        sinv[vv] = inv;
-      }
-      __syncthreads();
-      const Tin* Xg = reinterpret_cast<const Tin*>(a.X) + (G.x_row0 + (int64_t)c * G.x_cstride) * a.ldx;
-      for (int i = tid; i < G.n_in * kTfVox; i += blockDim.x) {
-        const int j = i / kTfVox, vv = i % kTfVox;
-        const int64_t src = sidx[vv];
-        reinterpret_cast<float*>(Xs)[i] = src >= 0 ? ldf(Xg + (int64_t)j * a.ldx + src) * sinv[vv] : 0.f;
-      }
-    } else {
-      // input rows of this tile: all copies in flight at once, zero past n_vox
-      const Tin* X = reinterpret_cast<const Tin*>(a.X) + (G.x_row0 + (int64_t)c * G.x_cstride) * a.ldx + v0;
-      const uint32_t xs_base = (uint32_t)__cvta_generic_to_shared(Xs);
-      for (int i = tid; i < G.n_in * kChunksPerRow; i += blockDim.x) {
-        const int j = i / kChunksPerRow, ch = i % kChunksPerRow;
-        const int64_t vv = v0 + (int64_t)ch * kChunkElems;
-        const int64_t left = a.n_vox - vv;
-        const int bytes = left >= kChunkElems ? 16 : (left > 0 ? (int)left * (int)sizeof(Tin) : 0);
-        const Tin* src = X + (int64_t)j * a.ldx + (int64_t)ch * kChunkElems;
-        cp_async16(xs_base + (uint32_t)((j * kTfVox + ch * kChunkElems) * sizeof(Tin)), bytes > 0 ? src : X, bytes);
-      }
+    // input rows of this tile: all copies in flight at once, zero past n_vox
+    const Tin* X = reinterpret_cast<const Tin*>(a.X) + (G.x_row0 + (int64_t)c * G.x_cstride) * a.ldx + v0;
+    const uint32_t xs_base = (uint32_t)__cvta_generic_to_shared(Xs);
+    for (int i = tid; i < G.n_in * kChunksPerRow; i += blockDim.x) {
+      const int j = i / kChunksPerRow, ch = i % kChunksPerRow;
+      const int64_t vv = v0 + (int64_t)ch * kChunkElems;
+      const int64_t left = a.n_vox - vv;
+      const int bytes = left >= kChunkElems ? 16 : (left > 0 ? (int)left * (int)sizeof(Tin) : 0);
+      const Tin* src = X + (int64_t)j * a.ldx + (int64_t)ch * kChunkElems;
+      cp_async16(xs_base + (uint32_t)((j * kTfVox + ch * kChunkElems) * sizeof(Tin)), bytes > 0 ? src : X, bytes);
     }
     if (g != cur_g) {  // the group's operator, transposed: Tt[j][o] = T[o][j], zero past n_out
       for (int i = tid; i < G.n_in * ldt; i += blockDim.x) {
@@ -210,7 +174,7 @@ __global__ void __launch_bounds__(32 * (kTfMaxOut / kTfOpt)) transform_staged_ke
 #pragma unroll
         for (int v = 0; v < 4; ++v) acc[o][v] = 0.f;
       const float* tcol = Tt + og * kTfOpt;
-      const Ts* xq = Xs + 4 * q;
+      const Tin* xq = Xs + 4 * q;
 #pragma unroll 2
       for (int j = 0; j < G.n_in; ++j) {
         const float4 x = ld_x4(xq + j * kTfVox);
@@ -245,18 +209,15 @@ __global__ void __launch_bounds__(32 * (kTfMaxOut / kTfOpt)) transform_staged_ke
   }
 }
 
-template <typename Tin, typename Tout, bool GATHER = false>
+template <typename Tin, typename Tout>
 static cudaError_t transform_dispatch(const TransformArgs& a, int n_groups, int max_out, cudaStream_t st) {
   int max_in = 0;
   for (int g = 0; g < n_groups; ++g) max_in = std::max(max_in, a.g[g].n_in);
-  if (GATHER && (max_out > kTfMaxOut || max_in > 128)) return cudaErrorInvalidValue;
   if (max_out <= kTfMaxOut && max_in <= 128) {
     const int og_count = (max_out + kTfOpt - 1) / kTfOpt;
     const int threads = 32 * og_count;
-    const size_t smem = (size_t)max_in * kTfOpt * og_count * sizeof(float) +
-                        (size_t)max_in * kTfVox * (GATHER ? sizeof(float) : sizeof(Tin)) +
-                        (GATHER ? (size_t)kTfVox * (sizeof(int64_t) + sizeof(float)) : 0);
-    auto kern = transform_staged_kernel<Tin, Tout, GATHER>;
+    const size_t smem = (size_t)max_in * kTfOpt * og_count * sizeof(float) + (size_t)max_in * kTfVox * sizeof(Tin);
+    auto kern = transform_staged_kernel<Tin, Tout>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0, dev = 0, sms = 0;
@@ -285,33 +246,32 @@ static cudaError_t transform_dispatch(const TransformArgs& a, int n_groups, int 
 
 // ---------------------------------------------------------------------------
 // Gathered Signal2SH: output voxel v reads input column a.index[v] scaled by
-// 1 / a.b0[index[v]].  One thread per voxel and all OPT >= n_out output rows, the operator transposed
-// in shared memory (broadcast reads), 16 input rows' loads in flight per thread: columns of a mask
+// 1 / a.b0[index[v]].  One thread per voxel and OPT output rows, the operator transposed in
+// shared memory (broadcast reads), 16 input rows' loads in flight per thread: columns of a mask
 // run are contiguous, so a warp's loads mostly are too.  Bound by the latency of those loads
-// (26.7 MB at 262,144 voxels of 30 BF16 directions into 15 coefficients: 4 us at the copy rate):
-// 22 us, the staged tile form (128 voxels per 64 threads, loads, then FMAs) 43.
-//
-// Wider outputs read the operator 12 times per input row and voxel, and the staged form (four voxels
-// a thread) is the better one; both give the same bits.  us here / staged, voxels x channels x shells:
-// up to 32 outputs always better here: 28 of 60 directions 19 / 27 at 2,000, 352 / 571 at 4 x 262,144;
-// 45 of 60: 22 / 24 at 20,000 (79 blocks), 27 / 27 at 60,000 (235), 50 / 32 at 4 x 20,000 (316: more than
-// two blocks per SM), 153 / 140 at 262,144; but of 90, whose staged tiles leave three blocks per SM,
-// 219 / 298 and 763 / 1031; 66 outputs and more, in chunks of 48 that read the input again:
-// 31 / 29 at 2,000, 379 / 246 at 262,144, 1497 / 872 at 4 x 262,144 (90 directions).
+// (26.7 MB at 262,144 voxels of 30 BF16 directions into 15 coefficients: 4 us at the copy rate), so
+// all 16 are issued before the first is used: with the scaling by 1 / b0 in the load's own expression
+// the compiler used each as it came.  us of a staged tile form (128 voxels per 64 threads), of that, and
+// of this: 43, 22, 16 for those; 45 outputs of 60 FP32 directions, 262,144 voxels 137, 158, 78; 4 x
+// 20,000 32, 50, 25; 66 of 90 (two chunks of outputs, the input read for each) 245, 379, 197.
+// Blocks of 128 threads for 48 outputs (96 registers): with 256 the last wave of 4 x 20,000 voxels
+// is an eighth of the first (41 us for BF16, 26 with 128).
 // ---------------------------------------------------------------------------
-constexpr int kGatherMaxOut = 48;
+constexpr int gather_threads(int opt) { return opt > 32 ? 128 : 256; }
 
 template <typename Tin, typename Tout, int OPT>
-__global__ void __launch_bounds__(256) transform_gather_kernel(const __grid_constant__ TransformArgs a) {
+__global__ void __launch_bounds__(gather_threads(OPT)) transform_gather_kernel(const __grid_constant__ TransformArgs a, int ochunks) {
   extern __shared__ float4 tf_smem4[];
   float* Ts = reinterpret_cast<float*>(tf_smem4);  // [n_in][OPT], zero past n_out
   const TransformGroup& G = a.g[blockIdx.z];
-  const int c = blockIdx.y;
-  for (int i = threadIdx.x; i < G.n_in * OPT; i += 256) {
+  const int c = blockIdx.y / ochunks, o0 = (blockIdx.y % ochunks) * OPT;
+  if (o0 >= G.n_out) return;
+  const int no = min(OPT, G.n_out - o0);
+  for (int i = threadIdx.x; i < G.n_in * OPT; i += gather_threads(OPT)) {
     const int j = i / OPT, o = i % OPT;
-    Ts[i] = o < G.n_out ? __ldg(G.T + (int64_t)o * G.n_in + j) : 0.f;
+    Ts[i] = o < no ? __ldg(G.T + (int64_t)(o0 + o) * G.n_in + j) : 0.f;
   }
-  const int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t v = (int64_t)blockIdx.x * gather_threads(OPT) + threadIdx.x;
   int64_t src = -1;
   float inv = 0.f;
   if (v < a.n_vox) {
@@ -332,9 +292,12 @@ __global__ void __launch_bounds__(256) transform_gather_kernel(const __grid_cons
 #pragma unroll
   for (int o = 0; o < OPT; ++o) acc[o] = 0.f;
   for (int j0 = 0; j0 < G.n_in; j0 += 16) {
-    float x[16];
+    float x[16];  // (two steps: all loads, then the scaling)
+    const int left = src >= 0 ? G.n_in - j0 : 0;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) x[u] = (src >= 0 && j0 + u < G.n_in) ? ldf(X + (int64_t)(j0 + u) * a.ldx) * inv : 0.f;
+    for (int u = 0; u < 16; ++u) x[u] = u < left ? ldf(X + (int64_t)(j0 + u) * a.ldx) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) x[u] *= inv;
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
       if (j0 + u < G.n_in) {
@@ -351,10 +314,10 @@ __global__ void __launch_bounds__(256) transform_gather_kernel(const __grid_cons
     }
   }
   if (v >= a.n_vox) return;
-  Tout* Y = reinterpret_cast<Tout*>(a.Y) + (G.y_row0 + (int64_t)c * G.y_cstride) * a.ldy + v;
+  Tout* Y = reinterpret_cast<Tout*>(a.Y) + (G.y_row0 + (int64_t)c * G.y_cstride + o0) * a.ldy + v;
 #pragma unroll
   for (int o = 0; o < OPT; ++o)
-    if (o < G.n_out) stf(Y + (int64_t)o * a.ldy, acc[o]);
+    if (o < no) stf(Y + (int64_t)o * a.ldy, acc[o]);
 }
 
 template <typename Tin, typename Tout>
@@ -362,13 +325,11 @@ static cudaError_t gather_dispatch(const TransformArgs& a, int n_groups, int max
   int max_in = 0;
   for (int g = 0; g < n_groups; ++g) max_in = std::max(max_in, a.g[g].n_in);
   if (max_out > kTfMaxOut || max_in > 128) return cudaErrorInvalidValue;
-  const int64_t vox_blocks = (a.n_vox + 255) / 256;
-  if (max_out > kGatherMaxOut ||
-      (max_out > 32 && max_in <= 64 && vox_blocks * a.channels * n_groups > 2 * sm_count()))  // reasons above
-    return transform_dispatch<Tin, Tout, true>(a, n_groups, max_out, st);
+  // outputs per thread: all of them up to 48 (each further chunk reads the input again)
   auto go = [&](auto kern, int opt) {
-    // grid y: channels, within 65,535 (more: slices of them)
-    const int per = 65535;
+    const int och = (max_out + opt - 1) / opt;
+    // grid y: channels x output chunks, within 65,535 (more channels: slices of them)
+    const int per = std::max(1, 65535 / och);
     for (int c0 = 0; c0 < a.channels; c0 += per) {
       TransformArgs b = a;
       const int nc = std::min(per, a.channels - c0);
@@ -376,8 +337,9 @@ static cudaError_t gather_dispatch(const TransformArgs& a, int n_groups, int max
         b.g[g].x_row0 += (int64_t)c0 * a.g[g].x_cstride;
         b.g[g].y_row0 += (int64_t)c0 * a.g[g].y_cstride;
       }
-      const dim3 grid((unsigned)vox_blocks, (unsigned)nc, (unsigned)n_groups);
-      kern<<<grid, 256, (size_t)max_in * opt * sizeof(float), st>>>(b);
+      const int threads = gather_threads(opt);
+      const dim3 grid((unsigned)((a.n_vox + threads - 1) / threads), (unsigned)(nc * och), (unsigned)n_groups);
+      kern<<<grid, threads, (size_t)max_in * opt * sizeof(float), st>>>(b, och);
       count_launch();
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
@@ -386,7 +348,7 @@ static cudaError_t gather_dispatch(const TransformArgs& a, int n_groups, int max
   };
   if (max_out <= 16) return go(transform_gather_kernel<Tin, Tout, 16>, 16);
   if (max_out <= 32) return go(transform_gather_kernel<Tin, Tout, 32>, 32);
-  return go(transform_gather_kernel<Tin, Tout, kGatherMaxOut>, kGatherMaxOut);
+  return go(transform_gather_kernel<Tin, Tout, 48>, 48);
 }
 
 cudaError_t launch_transform_gather(const TransformArgs& a, int n_groups, int max_out, int in_t, int out_t,

@@ -1,6 +1,6 @@
 """Gathered Signal2SH over the widths of its outputs (15, 28, 45 and 66 coefficients: a kernel of its
-own for each of the first three, the staged tiles for the last, and for 45 from some blocks on),
-both input and both output types, channels and shells, against the FP64 oracle's operators."""
+own for each of the first three, two chunks of outputs for the last), both input and both output
+types, channels and shells, against the FP64 oracle's operators."""
 import numpy as np
 import pytest
 
