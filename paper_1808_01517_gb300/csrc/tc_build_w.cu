@@ -7,7 +7,8 @@
 // TMEM): FP32-level accuracy before the result is rounded to BF16 (the same rounding point as
 // the CUDA-core build).  The parts of M are made once per geometry (M is fixed).
 //
-// What bounds it: the MMAs (144 of them per 128 pairs and four rows), close behind them writing
+// What bounds it: the thread that issues the MMAs (order 8, K = 49: 48 per tile of 128 pairs, four rows
+// and one input shell, about 100 cycles each whatever their width), close behind it writing
 // W (149 MB at 64 -> 64 channels, 29 MB at 16 -> 64).  One tile per CTA took 20 us, its loads,
 // MMAs, TMEM reads and stores one after the other; a persistent CTA that overlaps them, with
 // tiles of whole rows a so that every run of W leaves in one copy, measured 0.304 -> 0.083 ms
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) build_w_tc_kernel(const __grid_
     un.init(p, u0);
     int i = 0;
     for (int64_t u = u0; u < u1; ++u, ++i, un.next(p)) {
-      const bool valid = col < p.cpt && un.pt * p.cpt + col < d.c_out;
+      const bool valid = un.pt * p.cpt + col < d.c_out;
       bool ok = true;
       for (int hf = 0; hf < p.nh; ++hf) {
         ok = wait_bounded_sleep(stg_free(hf), (uint32_t)(i & 1) ^ 1u, abort_flag, p.err, kErrBwStgFree);
