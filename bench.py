@@ -31,12 +31,12 @@ METRIC = "voxels/s, Signal2SH->LSC->SH2Signal fwd+bwd, BF16 vs FP32 at stated er
 UNIT = "voxels/s"
 
 # DRAM traffic (read + write) of one launch at the 65,536-voxel workload, from the
-# single-pass ncu capture of the bench command summarised in
-# profiles/chain_65536vox_launch_list.md (the `dram__bytes_*` metrics); valid only
+# single-pass ncu capture of the bench command that the launch list under profiles/
+# summarises (the `dram__bytes_*` metrics); valid only
 # while the kernel's sources hash to the value recorded with the capture (re-hashed
-# only after host-side edits that leave the kernels' device code unchanged).
-_GEMM = ("csrc/tc_gemm.cu", "csrc/tc_ptx.cuh"), "2c9ebf18673e1755"
-_TF = ("csrc/tc_transform.cu", "csrc/tc_ptx.cuh"), "eb7c548664354ca4"
+# only after edits that leave the kernels' device code unchanged).
+_GEMM = ("csrc/tc_gemm.cu", "csrc/tc_ptx.cuh"), "b18b998e74774726"
+_TF = ("csrc/tc_transform.cu", "csrc/tc_ptx.cuh"), "945c6b1b222b7b42"
 NCU_TRAFFIC = {
     "lsc_fwd_gemm": {"bytes": 1.831e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},
     "lsc_dgrad_gemm": {"bytes": 3.479e9, "n_vox": 65536, "sources": _GEMM[0], "sha256_16": _GEMM[1]},

@@ -456,11 +456,14 @@ delimit_status delimit_selftest_wait_timeout(void* stream);
  *     before launching anything.
  *   0: every step on the CUDA-core kernels (same results within the dtype's
  *     rounding; used to cross-check the two).
- * Other values: INVALID_ARG.  The operator build runs on the tensor cores for
- * BF16 activations when K <= 64, c_in divides 128 and c_in * N_in is a multiple of 8
- * (modes 1 and 2), the weight gradient's reduction for BF16 activations when
- * K <= 64, else on the CUDA cores; they and the gathered Signal2SH are not counted
- * as fallbacks and never refused. */
+ * Other values: INVALID_ARG.  With modes 1 and 2 and BF16 activations, two smaller
+ * steps run on the tensor cores too where their kernels take the sizes, else on the
+ * CUDA cores: the operator build when K <= 64, c_in divides 128 and c_in * N_in is a
+ * multiple of 8; the weight gradient's reduction when K <= 64, N_out <= 128,
+ * min(128 / c_out, c_in) <= 32 (integer division, at least 0) and a part of the
+ * collapse matrices fits in shared memory (6 KiB per input coefficient of the part
+ * and 16 output coefficients; a part has about 256 of the N_out * N_in entries).
+ * They and the gathered Signal2SH are not counted as fallbacks and never refused. */
 delimit_status delimit_set_tensor_cores(int mode);
 
 /* Process-wide CTA-pair choice of the LSC tensor-core GEMMs (forward, input and

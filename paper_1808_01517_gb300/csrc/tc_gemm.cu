@@ -133,7 +133,10 @@ __device__ __forceinline__ uint32_t leaky_bf16x2(uint32_t x, uint32_t mask, floa
 // that 2 x 36 tiles do (64 -> 64 channels: an operator of 116 MB per 76 tiles), and the tiles of
 // one operator tile, equal in K, fill the rounds evenly.  64 -> 64 channels, 8,192 voxels: forward
 // 0.645 -> 0.589 ms, input gradient 0.654 -> 0.599 (groups of 4: 0.601 / 0.610, 32: 0.610 / 0.619);
-// 16 -> 64 channels, 65,536 voxels, where the operator fits L2: 1.240 -> 1.232 and 1.164 -> 1.168.
+// 16 -> 64 channels, 65,536 voxels, where the operator (37 MB) fits L2 and grouping saves nothing: 1.240 ->
+// 1.232 and 1.164 -> 1.168, at the cost of re-reads of the activations (DRAM reads of the forward 0.43 ->
+// 0.75 GB, of the input gradient 2.38 -> 3.21).  The rule below asks for K alone, not for the
+// operator's size.
 constexpr int kVoxGroup = 16;
 // up to this K a tile's time is its output's stores, not its operands: voxel tiles one by one
 constexpr int kShortK = 1024;

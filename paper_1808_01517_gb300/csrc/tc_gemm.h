@@ -36,9 +36,9 @@ void tc_basis_tables_destroy_f32(TcBasisTables& t);
 bool tc_transform_supported(const TcBasisTables& t, int kind, int64_t ldx, int64_t ldy, int out_t);
 cudaError_t tc_transform_launch(const TcBasisTables& t, int kind, const void* X, void* Y, int64_t n_vox, int C,
                                 int64_t ldx, int64_t ldy, int out_t, int* err_word, cudaStream_t st);
-// FP32 input (out_t: 0 = F32, 1 = BF16): each value split into three BF16 parts in shared
-// memory, six part products accumulated in FP32 on the tensor cores; aligned: X and its rows
-// start on 16-byte boundaries (else plain copies in place of TMA)
+// FP32 input (out_t: 0 = F32, 1 = BF16): each value split into three BF16 parts in registers,
+// stored to TMEM, six part products accumulated in FP32 on the tensor cores; aligned: X and its
+// rows start on 16-byte boundaries and come by TMA (else they are loaded into registers as they lie)
 bool tc_transform_f32_supported(const TcBasisTables& t, int kind, int out_t);
 cudaError_t tc_transform_f32_launch(const TcBasisTables& t, int kind, const float* X, void* Y, int64_t n_vox, int C,
                                     int64_t ldx, int64_t ldy, int out_t, bool aligned, int* err_word,
@@ -111,14 +111,15 @@ struct BuildWTables {
 cudaError_t build_w_tables_create(const LscDims& dims_template, const float* d_M, BuildWTables& t, std::string& err);
 void build_w_tables_destroy(BuildWTables& t);
 // The BF16 operator W on the tensor cores (zeros outside the window) and, where bias_vec is
-// given, the bias vector; K <= 64, c_in <= 128 and no padding between shell blocks.
+// given, the bias vector; K <= 64, c_in dividing 128 and no padding between shell blocks.
 bool tc_build_w_supported(const LscDims& d, const BuildWTables& t);
 cudaError_t tc_build_w(const LscDims& d, const BuildWTables& t, const float* w, const float* b, const float* q, void* W,
                        float* bias_vec, int* err, cudaStream_t st);
 
 // Parts of the collapse matrices for the weight gradient's reduction on the tensor cores: per
 // shell (or shell pair) and input coefficient b the three BF16 parts of M as operand images (ok
-// false: more than 64 kernel points or tables that do not fit; the CUDA-core reduction runs).
+// false: more than 64 kernel points, more than 128 output coefficients or images of a part beyond
+// shared memory; the CUDA-core reduction runs).
 struct ReduceDwTables {
   void* d_img = nullptr;
   int npg = 0;

@@ -13,8 +13,8 @@
 //
 // What bounds it: the thread that issues the MMAs, about 100 cycles each at these widths and 450 for
 // a group's wait and commit, then reading P (58 MB per split at 16 -> 64 channels, 232 MB at
-// 64 -> 64).  M's parts side by side in N make four MMAs of the six products of a k-step; six of them
-// with the same groups took 0.096 ms in the main kernel where this takes 0.092 (64 -> 64, one split).
+// 64 -> 64).  M's parts side by side in N make four MMAs of the six products of a k-step: 0.092 ms in the
+// main kernel (64 -> 64, one split; six MMAs, small ones first, in groups of four k-steps 0.096).
 // On the CUDA cores the step was bound by issue (64 FMAs per (b,a) entry and pair).  Measured, with
 // the sum of the parts and db: 64 -> 64 channels, one split 0.110 ms against 0.342 on the CUDA
 // cores, four splits 0.121 against 0.346; 16 -> 64 channels 0.035 and 0.047 against 0.095 and 0.100.

@@ -32,11 +32,16 @@
 // place of a copy of the input into padded rows: 30 directions of 3,658,350 voxels 0.183 ms against
 // 0.277 for the copy and 0.174 for the transform.  (4-byte cp.async into the ring took 0.324.)
 //
-// What bounds it: HBM.  With the parts written to shared memory for the MMA, shared-memory
-// bandwidth did: a 16 KiB chunk then cost 24 KiB of part writes and 48 KiB of A reads (each part
-// read by every product it enters) beside its own 32 KiB.  Through TMEM, Signal2SH of 450,000
-// voxels on 3 x 90 directions took 0.139 ms instead of 0.187, SH2Signal and its adjoint at
-// 262,144 voxels 0.162 ms instead of 0.194 together.
+// What bounds it: HBM at 450,000 voxels of 3 x 90 directions (Signal2SH at 78 % of copy), together with the
+// thread that issues the MMAs: a tile costs it about 100 cycles per MMA and 300 for each wait with
+// its fence and each commit, 1,450 for a tile of one chunk, which is what a call of few tiles takes.  With
+// the parts written to shared memory for the MMA, shared-memory bandwidth bound it: a 16 KiB chunk
+// then cost 24 KiB of part writes and 48 KiB of A reads (each part read by every product it enters)
+// beside its own 32 KiB.  Through TMEM, Signal2SH of 450,000 voxels on 3 x 90 directions took 0.139 ms
+// instead of 0.187, SH2Signal and its adjoint at 262,144 voxels 0.162 ms instead of 0.194 together.
+// Not every shape gained: SH2Signal of 64 directions from order 6 takes 119 us for 6 x 300,000 voxels
+// where the form through shared memory took 108 (three blocks to read per output; five to ten times
+// more exact), of 256 directions, with one accumulator, 47 us for 6 x 30,000 where it took 37.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
