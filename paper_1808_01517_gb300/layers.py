@@ -274,6 +274,48 @@ class _LSCFn(torch.autograd.Function):
         return d_in, dw, db, None, None, None, None, None
 
 
+class _LSCStackFn(torch.autograd.Function):
+    """LSC layers with a leaky ReLU between them in one node, activations and gradients as the
+    single layers make them; all its parameters' gradients arrive at its end."""
+
+    @staticmethod
+    def forward(ctx, x, slope, layers, *params):  # layers: (geom, c_in, c_out); params: w, b of each in turn
+        ctx.slope, ctx.layers = slope, layers
+        ctx.has_b = [b is not None for b in params[1::2]]
+        hs, ctx.ws = [x], []
+        for i, (geom, c_in, c_out) in enumerate(layers):
+            # a backward-sized workspace: the backward reuses the operator built here
+            ctx.ws.append(lsc_workspace(geom, x.shape[1], c_in, c_out, x.dtype, True, x.device))
+            hs.append(lsc_forward(geom, hs[-1], params[2 * i], params[2 * i + 1], c_in, c_out, workspace=ctx.ws[i],
+                                  slope=slope if i + 1 < len(layers) else None))
+        ctx.save_for_backward(*hs[:-1], *params[::2])
+        return hs[-1]
+
+    @staticmethod
+    def backward(ctx, g):
+        n = len(ctx.layers)
+        hs, ws = ctx.saved_tensors[:n], ctx.saved_tensors[n:]
+        grads = [None] * (2 * n)
+        for i in reversed(range(n)):
+            geom, c_in, c_out = ctx.layers[i]
+            need_x = i > 0 or ctx.needs_input_grad[0]
+            g, grads[2 * i], grads[2 * i + 1] = lsc_backward(
+                geom, hs[i], ws[i], g, c_in, c_out, need_input=need_x, need_weight=ctx.needs_input_grad[3 + 2 * i],
+                need_bias=ctx.has_b[i] and ctx.needs_input_grad[4 + 2 * i], workspace=ctx.ws[i],
+                operator_ready=ctx.ws[i] is not None, slope=ctx.slope if i > 0 else None)
+            ctx.ws[i] = None
+        return (g, None, None, *grads)
+
+
+def _followed(lscs) -> bool:
+    """Whether someone may wait for single parameters' gradients while a backward runs: hooks on them,
+    or a process group (a gradient exchange, whose hooks are not all to be seen from here)."""
+    dist = torch.distributed
+    return (dist.is_available() and dist.is_initialized()) or any(
+        p is not None and (p._backward_hooks or p._post_accumulate_grad_hooks)
+        for m in lscs for p in m._parameters.values())
+
+
 def _plain(m: torch.nn.Module, cls) -> bool:
     """m is exactly a cls and nothing watches or replaces its calls."""
     return type(m) is cls and "forward" not in m.__dict__ and not (
@@ -284,7 +326,9 @@ def _plain(m: torch.nn.Module, cls) -> bool:
 def lsc_stack(x: torch.Tensor, lscs, act) -> torch.Tensor:
     """lscs[-1](act(... act(lscs[0](x)))).  LSC layers and a LeakyReLU of this module on 2-D
     activations run with the leaky ReLU inside the layers' kernels; anything else (other modules,
-    subclasses, hooks on a module) is called as it is."""
+    subclasses, hooks on a module) is called as it is.  All layers' gradients arrive together, at the
+    end of the stack's backward, unless a parameter has a hook or a process group exists at the
+    forward: then layer by layer, each before the backward of the one below."""
     g = torch.nn.modules.module
     lscs = list(lscs)
     if not (x.dim() == 2 and len(lscs) > 1 and _plain(act, LeakyReLU)
@@ -294,16 +338,23 @@ def lsc_stack(x: torch.Tensor, lscs, act) -> torch.Tensor:
         for i, m in enumerate(lscs):
             x = m(x if i == 0 else act(x))
         return x
-    # a node per layer: a layer's gradients arrive, and what it kept is freed, before the next one's
-    # backward, as with the modules
-    slope_in = None
-    for i, m in enumerate(lscs):
-        w, b, slope = m.point_weights(), m.bias, act.slope if i + 1 < len(lscs) else None
-        if _untracked(x, w, b):  # no gradient flows through it: nothing is kept for a backward
-            x = lsc_forward(m.geom, x, w, b, m.c_in, m.c_out, slope=slope)
-        else:
-            x = _LSCFn.apply(x, w, b, m.geom, m.c_in, m.c_out, slope, slope_in)
-        slope_in = slope
+    params = [(m.point_weights(), m.bias) for m in lscs]
+    n, i = len(lscs), 0
+    while i < n and _untracked(x, *params[i]):  # layers that no gradient flows through keep nothing for a backward
+        m = lscs[i]
+        x = lsc_forward(m.geom, x, *params[i], m.c_in, m.c_out, slope=act.slope if i + 1 < n else None)
+        i += 1
+    if i == n:
+        return x
+    # A node per layer costs the host 30 us a layer and step (four layers of 16 channels at 512 voxels 0.77
+    # ms against 0.65), and is what lets a layer's gradients be used before the next one's backward.
+    if not _followed(lscs):
+        return _LSCStackFn.apply(x, act.slope, [(m.geom, m.c_in, m.c_out) for m in lscs[i:]],
+                                 *(p for wb in params[i:] for p in wb))
+    for k in range(i, n):
+        m = lscs[k]
+        x = _LSCFn.apply(x, *params[k], m.geom, m.c_in, m.c_out, act.slope if k + 1 < n else None,
+                         act.slope if k > i else None)
     return x
 
 

@@ -1,6 +1,7 @@
-"""Gradients of the network's stack of layers arrive layer by layer, last layer first, each before
-the backward of the layer below it runs (what overlaps a gradient exchange with the backward), and
-frozen layers are left out."""
+"""Gradients of the network's stack of layers, where hooks on the parameters or a process group may
+follow them, arrive layer by layer, last layer first, each before the backward of the layer below
+it runs (what overlaps a gradient exchange with the backward); frozen layers are left out; and both
+forms of the stack give the same bits."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -59,3 +60,31 @@ def test_frozen_layers(monkeypatch, frozen):
     events = _events(monkeypatch, m)
     m(x).float().square().sum().backward()
     assert [i for k, i in events if k == "backward"] == list(reversed(range(first, len(m.lscs))))
+
+
+def test_a_process_group_is_someone_who_follows(tmp_path):
+    """Data-parallel wrappers hook the gradients where the parameters do not show it."""
+    dist = torch.distributed
+    m, x = _net()
+
+    def nodes(y):
+        names, todo, seen = [], [y.grad_fn], set()
+        while todo:
+            f = todo.pop()
+            if f is not None and f not in seen:
+                seen.add(f)
+                names.append(type(f).__name__)
+                todo += [n for n, _ in f.next_functions]
+        return names.count("_LSCFnBackward"), names.count("_LSCStackFnBackward")
+
+    alone = m(x)
+    assert nodes(alone) == (0, 1)
+    want = torch.autograd.grad(alone.float().square().sum(), list(m.parameters()))
+    dist.init_process_group("gloo", init_method=f"file://{tmp_path}/store", rank=0, world_size=1)
+    try:
+        y = m(x)
+    finally:
+        dist.destroy_process_group()
+    assert nodes(y) == (len(m.lscs), 0)
+    got = torch.autograd.grad(y.float().square().sum(), list(m.parameters()))
+    assert torch.equal(y, alone) and all(torch.equal(a, b) for a, b in zip(got, want))
